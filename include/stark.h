@@ -45,11 +45,15 @@ extern "C" {
 #endif
 
 typedef enum {
-  STARK_F64 = 0,            /* fp64 in/out; fp64 leaves on CUDA cores                  */
+  STARK_F64 = 0,            /* fp64 in/out; leaves of side >= 128 as fp16 digit        */
+                            /* products on the tensor cores with an accuracy proof per  */
+                            /* product, redone on the CUDA cores where it fails; other  */
+                            /* leaves, depth-first and sharded plans on the CUDA cores  */
   STARK_F32_SPLIT_BF16 = 1, /* fp32 in/out; leaves as 3 bf16 products (hi*hi + hi*lo +  */
                             /* lo*hi, x = hi + lo) on tcgen05 tensor cores, fp32 accum. */
   STARK_F32_SPLIT_TF32 = 2, /* fp32 in/out; the same with TF32 halves                   */
-  STARK_I64 = 3,            /* int64 in/out; exact modulo 2^64 (two's complement)       */
+  STARK_I64 = 3,            /* int64 in/out; exact modulo 2^64 (two's complement); the  */
+                            /* same leaves                                              */
   STARK_F32_SPLIT_FP16 = 4  /* fp32 in/out; the same with IEEE fp16 halves (11 bits     */
                             /* each: about 22 bits per operand at the bf16 MMA rate).   */
                             /* Every leaf operand sum must stay below 65504 in         */

@@ -1,0 +1,143 @@
+// combine_limb.cu -- the combine of Alg. 5 for the F64 and I64 limb leaves as
+// an ordered pass over stored leaf products.
+//
+// A leaf product adds into up to 2^d quadrants of C.  As 64-bit reductions in
+// the leaf epilogue these came in bursts (all SMs end a tile together) at
+// 225 G/s for fp64, 33 us of every 150 us tile at n = 4096, depth 2, and
+// cleared C first; stored products cost 8 bytes per element instead, and this
+// pass reads them once and writes every element of C once.  A level takes its
+// additions as Alg. 1 writes them (C11 = M1 + M4 - M5 + M7, ...): 8 per four
+// elements, 5.5 per element of C at depth 2 against 9 by the expanded sums,
+// which matters because the SM adds two fp64 numbers a clock.
+//
+// One launch folds one or two levels; depths 3 and 4 take two launches, the
+// first into planes of the products two levels up.
+#include "stark_internal.h"
+
+namespace stark {
+namespace {
+
+template <typename T>
+struct Pair {
+  T x, y;
+};
+template <typename T>
+__device__ __forceinline__ Pair<T> operator+(const Pair<T>& a, const Pair<T>& b) {
+  return {a.x + b.x, a.y + b.y};
+}
+template <typename T>
+__device__ __forceinline__ Pair<T> operator-(const Pair<T>& a, const Pair<T>& b) {
+  return {a.x - b.x, a.y - b.y};
+}
+
+// Quadrants of a product from its seven sub-products.
+template <typename V>
+__device__ __forceinline__ void fold(const V (&m)[7], V (&c)[4]) {
+  c[0] = ((m[0] + m[3]) - m[4]) + m[6];
+  c[1] = m[2] + m[4];
+  c[2] = m[1] + m[3];
+  c[3] = ((m[0] - m[1]) + m[2]) + m[5];
+}
+
+// A thread owns two columns of one position (r, c) of the L x L leaf grid of
+// one product (blockIdx.y) D levels up: 7^D vectors in, 4^D out.
+template <typename T, int D>
+__global__ void __launch_bounds__(256, 2)
+    combine_limb_kernel(const T* __restrict__ M, int64_t L, T* __restrict__ out, int64_t out_plane, int64_t ld, int64_t n) {
+  using V = Pair<T>;
+  const int64_t pos = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  if (pos >= L * (L / 2)) return;
+  const int64_t r = pos / (L / 2), c = pos % (L / 2) * 2;
+  constexpr int P = D == 1 ? 7 : 49;
+  const T* src = M + (int64_t)blockIdx.y * P * L * L + r * L + c;
+  out += (int64_t)blockIdx.y * out_plane;
+  auto load = [&](int leaf) {
+    const int4 raw = __ldcs(reinterpret_cast<const int4*>(src + (int64_t)leaf * L * L));
+    return *reinterpret_cast<const V*>(&raw);
+  };
+  const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+  auto store = [&](int64_t row, int64_t col, const V& v) {
+    if (row >= n || col >= n) return;
+    T* dst = out + row * ld + col;
+    if (vec && col + 1 < n) {
+      *reinterpret_cast<int4*>(dst) = *reinterpret_cast<const int4*>(&v);
+    } else {
+      dst[0] = v.x;
+      if (col + 1 < n) dst[1] = v.y;
+    }
+  };
+  if constexpr (D == 1) {
+    V m[7], q[4];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) m[i] = load(i);
+    fold(m, q);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) store(r + (k >> 1) * L, c + (k & 1) * L, q[k]);
+  } else {
+    // the outer level's sums grow product by product, in Alg. 1's order
+    V s[16];
+#pragma unroll
+    for (int i = 0; i < 7; ++i) {
+      V m[7], q[4];
+#pragma unroll
+      for (int k = 0; k < 7; ++k) m[k] = load(i * 7 + k);
+      fold(m, q);
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        // M1: 11 22; M2: 21 -22; M3: 12 22; M4: 11 21; M5: -11 12; M6: 22; M7: 11
+        if (i == 0) s[k] = s[12 + k] = q[k];
+        if (i == 1) s[8 + k] = q[k], s[12 + k] = s[12 + k] - q[k];
+        if (i == 2) s[4 + k] = q[k], s[12 + k] = s[12 + k] + q[k];
+        if (i == 3) s[k] = s[k] + q[k], s[8 + k] = s[8 + k] + q[k];
+        if (i == 4) s[k] = s[k] - q[k], s[4 + k] = s[4 + k] + q[k];
+        if (i == 5) s[12 + k] = s[12 + k] + q[k];
+        if (i == 6) s[k] = s[k] + q[k];
+      }
+    }
+#pragma unroll
+    for (int o = 0; o < 4; ++o)
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        store(r + (2 * (o >> 1) + (k >> 1)) * L, c + (2 * (o & 1) + (k & 1)) * L, s[4 * o + k]);
+  }
+}
+
+template <typename T, int D>
+cudaError_t fold_levels(const T* M, int64_t L, int64_t products, T* out, int64_t out_plane, int64_t ld, int64_t n,
+                        cudaStream_t st) {
+  const int64_t blocks = (L * (L / 2) + 255) / 256;
+  if (L % 2 != 0 || blocks > 0x7FFFFFFF || products > 65535) return cudaErrorInvalidValue;
+  combine_limb_kernel<T, D><<<dim3((unsigned)blocks, (unsigned)products), 256, 0, st>>>(M, L, out, out_plane, ld, n);
+  count_launch();
+  return cudaGetLastError();
+}
+
+template <typename T>
+cudaError_t by_depth(const void* Mv, int depth, int64_t L, int64_t n, void* Cv, int64_t ldc, void* tmp, cudaStream_t st) {
+  const T* M = static_cast<const T*>(Mv);
+  T* C = static_cast<T*>(Cv);
+  T* mid = static_cast<T*>(tmp);
+  const int64_t side = 4 * L;
+  cudaError_t e;
+  switch (depth) {
+    case 1: return fold_levels<T, 1>(M, L, 1, C, 0, ldc, n, st);
+    case 2: return fold_levels<T, 2>(M, L, 1, C, 0, ldc, n, st);
+    case 3:
+      e = fold_levels<T, 2>(M, L, 7, mid, side * side, side, side, st);
+      return e != cudaSuccess ? e : fold_levels<T, 1>(mid, side, 1, C, 0, ldc, n, st);
+    case 4:
+      e = fold_levels<T, 2>(M, L, 49, mid, side * side, side, side, st);
+      return e != cudaSuccess ? e : fold_levels<T, 2>(mid, side, 1, C, 0, ldc, n, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+}  // namespace
+
+cudaError_t launch_combine_limb(const void* M, int depth, int64_t L, int64_t n, void* C, int64_t ldc, void* tmp,
+                                bool f64, cudaStream_t st) {
+  return f64 ? by_depth<double>(M, depth, L, n, C, ldc, tmp, st)
+             : by_depth<unsigned long long>(M, depth, L, n, C, ldc, tmp, st);
+}
+
+}  // namespace stark

@@ -64,6 +64,22 @@ __device__ __forceinline__ float rn_tf32(float x) {
   return __uint_as_float(u);
 }
 
+// x * 2^(62 - e) as an integer, rounded to nearest (ties away from zero), for
+// |x| <= 2^e; integer operations only.  e = kLimbZeroRow: x is zero.
+__device__ __forceinline__ unsigned long long fixed62(double x, int e) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
+  const int ex = (int)((bits >> 52) & 2047);
+  unsigned long long m = bits & 0xFFFFFFFFFFFFFull;
+  if (ex) m |= 0x10000000000000ull;
+  // |x| = m 2^(max(ex, 1) - 1075); zero rows shift to nothing
+  const int sh = e == kLimbZeroRow ? -64 : (ex ? ex : 1) - 1075 + 62 - e;
+  if (sh >= 0)
+    m <<= sh <= 10 ? sh : 10;
+  else
+    m = sh > -64 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull;
+  return (long long)bits < 0 ? 0ull - m : m;
+}
+
 // A short vector of accumulator values with elementwise + and -.
 template <typename Acc, int VEC>
 struct Vec {
@@ -90,10 +106,49 @@ struct Emitter {
   int64_t plane_elems;  // L * L
   int64_t offset;       // row * L + col of this thread's first element
   int* range_flag;
+  // digit planes of F64 operands
+  const int32_t* exps = nullptr;  // of leaf 0's row (side 0) or first column (side 1)
+  int64_t exp_leaf = 0;           // L
+  int exp_step = 0;               // 0: one exponent for the vector, 1: one per column
+  __half* mags = nullptr;         // null outside the first 128 of K
+  int64_t mag_leaf = 0;           // 128 L
 
   __device__ __forceinline__ void operator()(int leaf, const Vec<Acc, VEC>& x) const {
     const int64_t at = (int64_t)leaf * plane_elems + offset;
-    if constexpr (OUT == kOutBf16Exact) {
+    if constexpr (OUT == kOutLimbs) {
+      // the value as eight signed base-256 digits: the bytes of q + 0x80..80
+      // are the digits of q plus 128 each (mod 2^64, balanced); byte b becomes
+      // fp16 1024 + b by placing it under the exponent, and 1152 comes off
+      static_assert(VEC == 2, "two values per store");
+      unsigned long long q[2];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        if constexpr (std::is_same_v<Tin, double>)
+          q[e] = fixed62(x.v[e], exps[(int64_t)leaf * exp_leaf + e * exp_step]);
+        else
+          q[e] = (unsigned long long)x.v[e];
+        q[e] += 0x8080808080808080ull;
+      }
+      const int64_t base = ((int64_t)leaf * 8 * plane_elems + offset) / 2;
+      __half2* out = reinterpret_cast<__half2*>(hi) + base;
+#pragma unroll
+      for (int d = 0; d < 8; ++d) {
+        const int byte = std::is_same_v<Tin, double> ? 7 - d : d;  // F64: most significant digit first
+        const uint32_t w0 = (uint32_t)(q[0] >> (byte < 4 ? 0 : 32)), w1 = (uint32_t)(q[1] >> (byte < 4 ? 0 : 32));
+        // bytes (w0.b, 0x64, w1.b, 0x64) of the pair
+        const uint32_t sel = (uint32_t)(byte & 3) | ((uint32_t)(4 + (byte & 3)) << 4);
+        const uint32_t b = __byte_perm(w0, w1, sel);  // low half: byte of w0, byte of w1
+        const uint32_t h = __byte_perm(b, 0x64u, 0x4140u);
+        const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6480)));
+        __stcs(reinterpret_cast<unsigned int*>(out + d * (plane_elems / 2)), *reinterpret_cast<const unsigned int*>(&v));
+        if (d == 0 && std::is_same_v<Tin, double>) {
+          if (mags) {
+            const __half2 m = __habs2(v);
+            *reinterpret_cast<__half2*>(mags + (int64_t)leaf * mag_leaf) = m;
+          }
+        }
+      }
+    } else if constexpr (OUT == kOutBf16Exact) {
       // integer operand sums, exact in bf16 while |v| <= 256 (8 significant bits)
       __nv_bfloat16 h[VEC];
       bool bad = false;
@@ -297,7 +352,7 @@ struct Prefix {
 
 // K > 0: a depth-first subtree below K levels (input read through TopLoader).
 template <typename Tin, int OUT, int D, int SIDE, int VEC, int K>
-__global__ void __launch_bounds__(256, 2) divide_kernel(DivideArgs a, int vec_ok) {
+__device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
   using Acc = typename AccOf<Tin>::type;
   constexpr int R = D < 2 ? D : 2;  // levels done in registers
   constexpr int F = D - R;          // levels walked as an outer loop
@@ -321,12 +376,50 @@ __global__ void __launch_bounds__(256, 2) divide_kernel(DivideArgs a, int vec_ok
   } else {
     ld = ld0;
   }
-  const Emitter<OUT, Tin, VEC> emit{a.out_hi, a.out_lo, a.L * a.L, i * a.L + j, a.range_flag};
+  Emitter<OUT, Tin, VEC> emit{a.out_hi, a.out_lo, a.L * a.L, i * a.L + j, a.range_flag};
+  if constexpr (OUT == kOutLimbs && std::is_same_v<Tin, double>) {
+    emit.exps = a.exps + (SIDE == 0 ? i : j);
+    emit.exp_leaf = a.L;
+    emit.exp_step = SIDE;
+    emit.mag_leaf = kLimbCheckK * a.L;
+    __half* mags = static_cast<__half*>(a.mags);
+    if (SIDE == 0)
+      emit.mags = j < kLimbCheckK ? mags + i * kLimbCheckK + j : nullptr;
+    else
+      emit.mags = i < kLimbCheckK ? mags + i * a.L + j : nullptr;
+  }
   const int64_t npad = a.npad;
 
   auto leaf_block = [&](const int* dig, int prefix) {
     // the 4^R sub-quadrant vectors below this prefix, then the register tree
     Vec<Acc, VEC> in[pow4c(R)];
+    if constexpr (F == 1 && OUT == kOutLimbs) {
+      // one outer level: its second terms are loaded after all the first
+      // ones, so that sixteen loads are in flight at a time
+      const TermPair t = terms_of<SIDE>(dig[0]);
+      const int64_t h = npad >> 1;
+      auto at = [&](int g, int q) {
+        int64_t r = i + (q >> 1) * h, c = j + (q & 1) * h;
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+          const int digit = (g >> (2 * (R - 1 - k))) & 3;
+          r += (int64_t)(digit >> 1) * (npad >> (F + k + 1));
+          c += (int64_t)(digit & 1) * (npad >> (F + k + 1));
+        }
+        return ld(r, c);
+      };
+#pragma unroll
+      for (int g = 0; g < pow4c(R); ++g) in[g] = at(g, t.qa);
+      if (t.qb >= 0) {
+#pragma unroll
+        for (int g = 0; g < pow4c(R); ++g) {
+          const Vec<Acc, VEC> w = at(g, t.qb);
+          in[g] = t.sb > 0 ? in[g] + w : in[g] - w;
+        }
+      }
+      Tree<Acc, SIDE, R, VEC>::run(in, prefix, emit);
+      return;
+    }
 #pragma unroll
     for (int g = 0; g < pow4c(R); ++g) {
       int64_t r = i, c = j;
@@ -357,6 +450,12 @@ __global__ void __launch_bounds__(256, 2) divide_kernel(DivideArgs a, int vec_ok
     }
     leaf_block(dig, p);
   }
+}
+
+template <typename Tin, int OUT, int D, int SIDE, int VEC, int K>
+__global__ void __launch_bounds__(256, 2) divide_kernel(DivideArgs a, int vec_ok) {
+  if (a.gate && *(volatile const int*)a.gate == 0) return;
+  divide_body<Tin, OUT, D, SIDE, VEC, K>(a, vec_ok);
 }
 
 template <typename Tin, int OUT, int D, int SIDE, int K>

@@ -1,0 +1,157 @@
+// limb_bounds.cu -- what the F64 limb leaves need before their divide: for
+// every leaf operand row of A and column of B an exponent e with |x| <= 2^e
+// for all its elements, and the flag that sends a product to the CUDA cores.
+//
+// The bound comes from the inputs, not from the operand sums: one read of A
+// and B gives the largest magnitude of every row (column) within every
+// quadrant column (row) block of the deepest level, and a leaf's bound is the
+// sum of its quadrants' maxima in the order of the divide's own additions, so
+// by monotonicity of rounding no rounded operand sum exceeds it.  The read is
+// bound by HBM; reducing the operand sums themselves would read them 7/4
+// times per level instead of once.
+#include "divide_impl.cuh"
+
+namespace stark {
+namespace {
+
+// Magnitude bits: integer order is magnitude order, NaN above infinity.
+__device__ __forceinline__ unsigned long long mag_bits(double x) {
+  return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+}
+
+// blockIdx.z == 0: a warp takes one row of A in one column block; 1: a block
+// takes 32 columns of B in one row block.  Rows and columns beyond n are zero.
+__global__ void __launch_bounds__(256) limb_max_kernel(LimbBoundsArgs a) {
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int blocks = 1 << a.depth;
+  const int64_t L = a.L;
+  if (blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 0) *a.flag = 0;
+  if (blockIdx.z == 0) {
+    for (int64_t u = (int64_t)blockIdx.x * 8 + warp; u < a.npad * blocks; u += (int64_t)gridDim.x * 8) {
+      const int64_t row = u / blocks, q = u % blocks;
+      unsigned long long m = 0;
+      if (row < a.n) {
+        const int64_t c1 = (q + 1) * L < a.n ? (q + 1) * L : a.n;
+        const double* p = a.A + row * a.ld;
+        int64_t c = q * L + lane;
+        for (; c + 96 < c1; c += 128) {
+          const unsigned long long x0 = mag_bits(p[c]), x1 = mag_bits(p[c + 32]), x2 = mag_bits(p[c + 64]),
+                                   x3 = mag_bits(p[c + 96]);
+          m = max(m, max(max(x0, x1), max(x2, x3)));
+        }
+        for (; c < c1; c += 32) m = max(m, mag_bits(p[c]));
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if (lane == 0) a.max_a[q * a.npad + row] = __longlong_as_double((long long)m);
+    }
+  } else {
+    __shared__ unsigned long long part[8][32];
+    const int64_t groups = a.npad / 32;
+    for (int64_t u = blockIdx.x; u < groups * blocks; u += gridDim.x) {
+      const int64_t col = u % groups * 32 + lane, q = u / groups;
+      const int64_t r1 = (q + 1) * L < a.n ? (q + 1) * L : a.n;
+      unsigned long long m = 0;
+      if (col < a.n) {
+        const double* p = a.B + col;
+        int64_t r = q * L + warp;
+        for (; r + 56 < r1; r += 64) {
+          unsigned long long x[8];
+#pragma unroll
+          for (int e = 0; e < 8; ++e) x[e] = mag_bits(p[(r + 8 * e) * a.ld]);
+#pragma unroll
+          for (int e = 0; e < 8; ++e) m = max(m, x[e]);
+        }
+        for (; r < r1; r += 8) m = max(m, mag_bits(p[r * a.ld]));
+      }
+      part[warp][lane] = m;
+      __syncthreads();
+      if (warp == 0) {
+#pragma unroll
+        for (int w = 1; w < 8; ++w) m = max(m, part[w][lane]);
+        a.max_b[q * a.npad + col] = __longlong_as_double((long long)m);
+      }
+      __syncthreads();
+    }
+  }
+}
+
+// One thread per (leaf, row of A) and (leaf, column of B).
+__global__ void __launch_bounds__(256) limb_exp_kernel(LimbBoundsArgs a, int64_t leaves) {
+  const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  const int side = blockIdx.y;
+  if (t >= leaves * a.L) return;
+  const int leaf = (int)(t / a.L);
+  const int64_t i = t % a.L;  // row (side 0) or column (side 1) of the leaf
+  const double* mx = side == 0 ? a.max_a : a.max_b;
+  int dig[4] = {0, 0, 0, 0};
+  int x = leaf;
+  for (int k = a.depth - 1; k >= 0; --k) {
+    dig[k] = x % 7;
+    x /= 7;
+  }
+  // the divide adds level by level, the last level outermost: term u (bit k:
+  // second term of level k + 1), folded pairwise from the top level down
+  double v[16];
+  const int terms = 1 << a.depth;
+  for (int u = 0; u < terms; ++u) {
+    int64_t row = 0, col = 0;
+    bool present = true;
+    for (int k = 0; k < a.depth; ++k) {
+      const TermPair tp = side == 0 ? terms_of<0>(dig[k]) : terms_of<1>(dig[k]);
+      const int second = (u >> k) & 1;
+      const int q = second ? tp.qb : tp.qa;
+      if (q < 0) {
+        present = false;
+        break;
+      }
+      row += (int64_t)(q >> 1) * (a.npad >> (k + 1));
+      col += (int64_t)(q & 1) * (a.npad >> (k + 1));
+    }
+    v[u] = 0.0;
+    if (present) v[u] = side == 0 ? mx[col / a.L * a.npad + row + i] : mx[row / a.L * a.npad + col + i];
+  }
+  // S_1 sums pairs that differ in bit 0 (the top level), S_2 in bit 1, ...
+  for (int k = 0, w = terms / 2; k < a.depth; ++k, w /= 2)
+    for (int u = 0; u < w; ++u) v[u] = v[2 * u] + v[2 * u + 1];
+  const unsigned long long b = mag_bits(v[0]);
+  int32_t e = kLimbZeroRow;
+  if (b != 0) {
+    const int ex = (int)(b >> 52);
+    e = ex - 1023 + ((b & 0xFFFFFFFFFFFFFull) ? 1 : 0);  // smallest e with bound <= 2^e (normal numbers)
+    if (ex == 2047 || e < -400 || e > 400) {
+      *(volatile int*)a.flag = 1;
+      e = 0;  // (any value: the product is redone)
+    }
+  }
+  (side == 0 ? a.expA : a.expB)[t] = e;
+}
+
+__global__ void __launch_bounds__(256) gated_clear_kernel(unsigned long long* C, int64_t n, int64_t ld, const int* gate) {
+  if (*(volatile const int*)gate == 0) return;
+  for (int64_t r = blockIdx.x; r < n; r += gridDim.x)
+    for (int64_t c = threadIdx.x; c < n; c += 256) C[r * ld + c] = 0ull;
+}
+
+}  // namespace
+
+cudaError_t launch_limb_bounds(const LimbBoundsArgs& a, cudaStream_t st) {
+  int64_t leaves = 1;
+  for (int k = 0; k < a.depth; ++k) leaves *= 7;
+  const int64_t units = a.npad << a.depth;  // rows of A; a block of 8 warps or 32 columns of B per 8 of them
+  const int64_t blocks = (units + 31) / 32;
+  limb_max_kernel<<<dim3((unsigned)(blocks < 2432 ? blocks : 2432), 1, 2), 256, 0, st>>>(a);
+  count_launch();
+  const int64_t t = leaves * a.L;
+  limb_exp_kernel<<<dim3((unsigned)((t + 255) / 256), 2), 256, 0, st>>>(a, leaves);
+  count_launch();
+  return cudaGetLastError();
+}
+
+cudaError_t launch_gated_clear(void* C, int64_t n, int64_t ld, const int* gate, int num_sms, cudaStream_t st) {
+  gated_clear_kernel<<<(unsigned)(4 * num_sms), 256, 0, st>>>(static_cast<unsigned long long*>(C), n, ld, gate);
+  count_launch();
+  return cudaGetLastError();
+}
+
+}  // namespace stark

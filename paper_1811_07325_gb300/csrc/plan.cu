@@ -131,6 +131,19 @@ bool make_tmap_mplanes(CUtensorMap* m, void* base, int64_t L, int64_t planes) {
   return r == CUDA_SUCCESS;
 }
 
+bool make_tmap_half3(CUtensorMap* m, void* base, int64_t cols, int64_t rows, int64_t planes, int box_cols, int box_rows,
+                     int box_planes) {
+  auto fn = encode_fn();
+  if (!fn) return false;
+  cuuint64_t dims[3] = {(cuuint64_t)cols, (cuuint64_t)rows, (cuuint64_t)planes};
+  cuuint64_t strides[2] = {(cuuint64_t)(cols * 2), (cuuint64_t)(cols * rows * 2)};
+  cuuint32_t box[3] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows, (cuuint32_t)box_planes};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  box_cols == 64 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
 bool make_tmap_c(CUtensorMap* m, void* C, int64_t n, int64_t ld) {
   auto fn = encode_fn();
   if (!fn || n <= 0 || ld < n || (ld % 4) != 0 || (reinterpret_cast<uintptr_t>(C) & 15) != 0) return false;
@@ -242,6 +255,56 @@ double model_seconds(int64_t n, int depth, stark_dtype dt) {
   return flops / rate * waves + (in_bytes + ws + c_bytes) / 6.7e12 + launches * 22e-6 + 5e-6;
 }
 
+// Whether a product of this plan runs its leaves as digit products.
+static bool plan_limbs(const stark_plan_s* p) {
+  return p->limb_ok && !p->int_tc && !p->dfs && !p->shard_levels && p->op_elem == 16;
+}
+
+// Tensor maps of the digit planes.
+static bool plan_limb_maps(stark_plan_s* p) {
+  // A: four planes of 128 rows x 32 of K; B: four of 32 of K x 64 columns
+  bool ok = make_tmap_half3(&p->tmLA, p->X, p->L, p->L, p->P * 8, 32, 128, 4) &&
+            make_tmap_half3(&p->tmLB, p->Y, p->L, p->L, p->P * 8, 64, 32, 4);
+  if (p->dt == STARK_F64)
+    ok = ok && make_tmap_half3(&p->tmSA, p->mag_a, kLimbCheckK, p->L, p->P, 32, 128, 1) &&
+         make_tmap_half3(&p->tmSB, p->mag_b, p->L, kLimbCheckK, p->P, 64, 32, 1);
+  return ok;
+}
+
+// The same for a plan that may run limb leaves (leaf side >= 128): rounds of
+// 128 x 128 tiles over the SMs, each costing its 128-deep superchunks and a
+// share of its end, and the traffic of the divide (16 bytes written per
+// operand element), of the stored products and of the inputs and C at the
+// rates the passes reach (the deep F64 divides are bound by their fp64
+// additions, two a clock and SM).  Constants measured on GB300 at n = 200 to
+// 8192, depths 0 to 3; every pick there is within 6 % of the fastest depth.
+static double plan_seconds(int64_t n, int depth, stark_dtype dt) {
+  const int64_t npad = padded_side(n, depth, dt), L = npad >> depth;
+  if (L < 128) return model_seconds(n, depth, dt);
+  const bool f64 = dt == STARK_F64;
+  int dev = 0, v = 0;
+  const bool have = cudaGetDevice(&dev) == cudaSuccess &&
+                    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess && v > 0;
+  cudaGetLastError();
+  const double P = (double)pow7i(depth), side = std::ceil(L / 128.0), sms = have ? (double)v : 152.0;
+  const double rounds = std::ceil(P * side * side / sms), chunks = L / 128.0;
+  const double leaf = f64 ? rounds * (chunks * 16.0e-6 + 6e-6) + 40e-6 : rounds * (chunks * 14.8e-6 + 3e-6) + 19e-6;
+  const double bytes = P * L * L * (depth ? 48.0 : 32.0) + (double)n * n * (f64 ? 40.0 : 24.0);
+  const double rate = f64 ? (depth <= 1 ? 5.0e12 : depth == 2 ? 3.3e12 : 2.2e12) : (depth <= 1 ? 6.0e12 : 4.6e12);
+  return leaf + bytes / rate;
+}
+
+int choose_plan_depth(int64_t n, stark_dtype dt) {
+  int best = 0;
+  double best_t = 1e300;
+  for (int d = 0; d <= 3; ++d)
+    if (const double t = plan_seconds(n, d, dt); t < best_t) {
+      best_t = t;
+      best = d;
+    }
+  return best;
+}
+
 int choose_depth(int64_t n, stark_dtype dt) {
   int best = 0;
   double best_t = 1e300;
@@ -304,7 +367,7 @@ stark_status stark_plan_ex(int64_t n, int depth, stark_dtype dt, unsigned flags,
   if (dt != STARK_F64 && dt != STARK_I64 && !is_split(dt)) return STARK_EINVAL;
   if (n > (int64_t)1 << 20) return STARK_EINVAL;
   if (!device_is_sm100_family()) return STARK_EUNSUPPORTED;
-  if (depth < 0) depth = is_split(dt) ? autotune_depth(n, dt) : choose_depth(n, dt);
+  if (depth < 0) depth = is_split(dt) ? autotune_depth(n, dt) : choose_plan_depth(n, dt);
   auto* p = new (std::nothrow) stark_plan_s();
   if (!p) return STARK_ENOMEM;
   stark_status st = plan_init(p, n, depth, dt, (flags & STARK_PLAN_PEEL) != 0);
@@ -339,8 +402,9 @@ stark_status stark_plan_get_info(stark_plan_t p, stark_plan_info* info) {
   info->dtype = p->dt;
   info->leaves = p->P;
   info->workspace_bytes = p->ws_bytes;
-  info->tile_m = p->is_tc ? 128 : 64;
-  info->tile_n = p->is_tc ? p->bn : 64;
+  const bool limbs = plan_limbs(p);
+  info->tile_m = p->is_tc || limbs ? 128 : 64;
+  info->tile_n = p->is_tc ? p->bn : limbs ? 128 : 64;
   info->combine = p->combine_mode;
   info->shard_levels = p->shard_levels;
   info->shard_first = (int32_t)p->shard_first;
@@ -580,10 +644,11 @@ static stark_status plan_tune_combine(stark_plan_t p) {
 
 // Workspace for `planes_per_half` leaves per operand side, with its maps.
 static stark_status plan_alloc_operands(stark_plan_s* p, int64_t planes) {
-  const int64_t per = half_split(p->dt) ? 4 : 8;  // bytes per leaf element per operand
+  // bytes per leaf element per operand (digit planes: only breadth first)
+  const int64_t per = half_split(p->dt) ? 4 : p->limb_ok && planes == p->P ? 16 : 8;
   const int64_t bytes = planes * p->L * p->L * per;
   if (cudaDeviceSynchronize() != cudaSuccess) return STARK_ECUDA;
-  const int64_t old = p->P_ws * p->L * p->L * per;
+  const int64_t old = p->P_ws * p->L * p->L * p->op_elem;
   // the new workspace first, so that on failure the plan keeps the old one;
   // when shrinking on a nearly full device, release the old one first
   void* X = nullptr;
@@ -615,6 +680,8 @@ static stark_status plan_alloc_operands(stark_plan_s* p, int64_t planes) {
   p->Y = Y;
   p->ws_bytes += 2 * bytes;
   p->P_ws = planes;
+  p->op_elem = per;
+  if (per == 16 && !plan_limb_maps(p)) return STARK_EUNSUPPORTED;
   if (stark_status st = plan_operand_maps(p, planes); st != STARK_OK) return st;
   if (p->int_tc && (!make_tmap_planes(&p->tmAi, p->X, false, p->L, planes, 128) ||
                     !make_tmap_planes(&p->tmBi, p->Y, false, p->L, planes, 64)))
@@ -802,7 +869,82 @@ bool traversal_supported(int depth, stark_dtype dt, int levels) {
   return levels == 1 || is_split(dt);
 }
 
-stark_status plan_init(stark_plan_s* p, int64_t n, int depth, stark_dtype dt, bool peel, int dfs) {
+// The magnitude sum each F64 leaf's elements must reach (leaf_limb.cu has the
+// derivation), from the leaf side and the terms that padding leaves the leaf.
+static void limb_check_sums(const stark_plan_s* p, std::vector<float>& need) {
+  const double rounded = p->L <= 1024 ? 1.0 : 1.5;  // half units a superchunk
+  const double full = 16384.0 * (1.0 / 64 + rounded * (double)p->L / 128.0 / 512.0);
+  const float full_need = (float)std::max(512.0, full);
+  need.assign((size_t)p->P, full_need);
+  if (p->depth == 0) return;
+  std::vector<int64_t> terms((size_t)p->P, kLimbCheckK);
+  for (int side = 0; side < 2; ++side) {
+    std::vector<int32_t> cnt, quad;
+    std::vector<int8_t> sign;
+    build_quadrant_table(p->depth, side, cnt, quad, sign);
+    for (int64_t l = 0; l < p->P; ++l) {
+      int64_t k = 0;  // K positions with an input element in some term (columns of A, rows of B)
+      for (int t = 0; t < cnt[(size_t)l]; ++t) {
+        int64_t r = 0, c = 0;
+        quadrant_offsets(p->depth, p->npad, quad[(size_t)(l << p->depth) + t], &r, &c);
+        k = std::max(k, core_side(p) - (side == 0 ? c : r));
+      }
+      terms[(size_t)l] = std::min(terms[(size_t)l], k);
+    }
+  }
+  for (int64_t l = 0; l < p->P; ++l)
+    if (terms[(size_t)l] < kLimbCheckK) need[(size_t)l] = terms[(size_t)l] < 16 ? 0.f : (float)terms[(size_t)l];
+}
+
+// X and Y for the digit planes (`ws` bytes together) and, for F64, the bounds,
+// exponents and magnitude planes with the flag.  On failure nothing is kept.
+static bool plan_limb_alloc(stark_plan_s* p, int64_t ws) {
+  bool ok = cudaMalloc(&p->X, (size_t)(ws / 2)) == cudaSuccess && cudaMalloc(&p->Y, (size_t)(ws / 2)) == cudaSuccess;
+  int64_t aux = 0, products = 0;
+  if (ok && p->depth > 0) {
+    products = p->P * p->L * p->L * 8;
+    ok = cudaMalloc(&p->limb_m, (size_t)products) == cudaSuccess;
+  }
+  if (ok && p->dt == STARK_F64) {
+    const int64_t maxima = (p->npad << p->depth) * 8, exps = (p->P * p->L * 4 + 255) / 256 * 256,
+                  mags = p->P * p->L * kLimbCheckK * 2;
+    const int64_t needs = (p->P * 4 + 255) / 256 * 256;
+    aux = 256 + needs + 2 * (maxima + exps + mags);
+    ok = cudaMalloc(&p->limb_aux, (size_t)aux) == cudaSuccess;
+    if (ok) {
+      char* b = static_cast<char*>(p->limb_aux);
+      p->d_flag = reinterpret_cast<int*>(b);
+      b += 256;  // every part is a multiple of 256 bytes
+      p->limb_need = reinterpret_cast<float*>(b);
+      b += needs;
+      p->mag_a = b;
+      p->mag_b = b + mags;
+      b += 2 * mags;
+      p->exp_a = reinterpret_cast<int32_t*>(b);
+      p->exp_b = reinterpret_cast<int32_t*>(b + exps);
+      b += 2 * exps;
+      p->max_a = reinterpret_cast<double*>(b);
+      p->max_b = reinterpret_cast<double*>(b + maxima);
+      std::vector<float> need;
+      limb_check_sums(p, need);
+      ok = cudaMemcpy(p->limb_need, need.data(), need.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+    }
+  }
+  ok = ok && plan_limb_maps(p);
+  if (ok) {
+    p->ws_bytes += aux + products;
+    return true;
+  }
+  cudaGetLastError();
+  cudaFree(p->X);
+  cudaFree(p->Y);
+  cudaFree(p->limb_m);
+  cudaFree(p->limb_aux);
+  p->X = p->Y = p->limb_m = p->limb_aux = nullptr;
+  return false;
+}
+
+stark_status plan_init(stark_plan_s* p, int64_t n, int depth, stark_dtype dt, bool peel, int dfs, bool lean) {
   if (!traversal_supported(depth, dt, dfs)) return STARK_EUNSUPPORTED;
   p->n = n;
   p->depth = depth;
@@ -822,12 +964,19 @@ stark_status plan_init(stark_plan_s* p, int64_t n, int depth, stark_dtype dt, bo
   p->num_sms = device_sm_count();
   if (p->L > 0x7FFFFFFF / 2) return STARK_EINVAL;
 
-  const int64_t ws = operand_bytes(core, depth, dt) / pow7i(dfs);
-  if (cudaMalloc(&p->X, (size_t)(ws / 2)) != cudaSuccess || cudaMalloc(&p->Y, (size_t)(ws / 2)) != cudaSuccess) {
+  int64_t ws = operand_bytes(core, depth, dt) / pow7i(dfs);
+  p->op_elem = half_split(dt) ? 4 : 8;
+  // digit planes take 16 bytes per element; where they or the F64 side arrays
+  // do not fit, the plan runs on the CUDA cores as a lean one does
+  p->limb_ok = !p->is_tc && !lean && dfs == 0 && p->L >= 128 && plan_limb_alloc(p, 2 * ws);
+  if (p->limb_ok) {
+    ws *= 2;
+    p->op_elem = 16;
+  } else if (cudaMalloc(&p->X, (size_t)(ws / 2)) != cudaSuccess || cudaMalloc(&p->Y, (size_t)(ws / 2)) != cudaSuccess) {
     cudaGetLastError();
     return STARK_ENOMEM;
   }
-  p->ws_bytes = ws;
+  p->ws_bytes += ws;
 
   // C targets of every leaf (side 2 of the quadrant-index table)
   std::vector<int32_t> cnt, quad;
@@ -902,6 +1051,8 @@ void plan_release(stark_plan_s* p) {
   cudaFree(p->cstage);
   cudaFree(p->m_planes);
   cudaFree(p->q_planes);
+  cudaFree(p->limb_m);
+  cudaFree(p->limb_aux);
   for (auto e : p->ev)
     if (e) cudaEventDestroy(e);
   p->ev.clear();
@@ -1016,10 +1167,17 @@ static bool plan_sib(const stark_plan_s* p, int64_t lb, int64_t le) {
          (half_split(p->dt) || p->tf32_mn);
 }
 
-// Whether a separate pass writes every element of C (combine modes 2 and 3):
+// Whether the limb leaves of [lb, le) are stored and combined by an ordered
+// pass (a whole product), not added into C by the leaf kernel.
+static bool plan_limb_stored(const stark_plan_s* p, int64_t lb, int64_t le) {
+  return plan_limbs(p) && lb == 0 && le == p->P;
+}
+
+// Whether a separate pass writes every element of C (combine modes 2 and 3,
+// limb leaves):
 // then C is not cleared first and no staging copy is used.
 static bool plan_stored(const stark_plan_s* p, int64_t lb, int64_t le) {
-  return plan_deterministic(p, lb, le) || plan_sib(p, lb, le);
+  return plan_deterministic(p, lb, le) || plan_sib(p, lb, le) || plan_limb_stored(p, lb, le);
 }
 
 // Leaf products of leaves [lb, le) with the combine, operands in workspace
@@ -1141,6 +1299,80 @@ static stark_status plan_leaves(stark_plan_s* p, void* C, int64_t lb, int64_t le
   return st;
 }
 
+// Digit planes of every leaf operand (I64, F64), for F64 after the bounds.
+static stark_status plan_limb_divide(stark_plan_s* p, const void* A, const void* B, cudaStream_t s) {
+  DivideArgs da{A, core_side(p), p->npad, p->L, p->X, nullptr, p->d_err, -1, p->n};
+  DivideArgs db{B, core_side(p), p->npad, p->L, p->Y, nullptr, p->d_err, -1, p->n};
+  if (p->dt == STARK_F64) {
+    const LimbBoundsArgs b{static_cast<const double*>(A), static_cast<const double*>(B), core_side(p), p->n, p->npad,
+                           p->L, p->depth, p->max_a, p->max_b, p->exp_a, p->exp_b, p->d_flag};
+    if (stark_status st = to_status(launch_limb_bounds(b, s)); st != STARK_OK) return st;
+    da.exps = p->exp_a;
+    db.exps = p->exp_b;
+    da.mags = p->mag_a;
+    db.mags = p->mag_b;
+  }
+  return to_status(launch_divide_limbs(da, db, p->depth, p->dt == STARK_F64 ? kInF64 : kInI64, s));
+}
+
+// Their products, combined into C.  F64: followed by the same range of leaves
+// on the CUDA cores, launches that do nothing unless the device flag says that
+// some element's accuracy is not proven (C then starts from zero again).
+static stark_status plan_limb_leaves(stark_plan_s* p, const void* A, const void* B, void* C, int64_t lb, int64_t le,
+                                     cudaStream_t s) {
+  const bool f64 = p->dt == STARK_F64;
+  LeafLimbArgs a{};
+  a.L = (int32_t)p->L;
+  a.leaf_begin = (int32_t)lb;
+  a.leaf_end = (int32_t)le;
+  a.ctab = p->d_ctab;
+  a.ccount = p->d_ccount;
+  a.maxT = p->maxT;
+  a.C = C;
+  a.ldc = p->n;
+  a.n = core_side(p);
+  const bool stored = plan_limb_stored(p, lb, le);
+  a.store = !stored ? nullptr : p->depth ? p->limb_m : C;
+  a.err = p->d_err;
+  a.timeout_ns = p->timeout_ns;
+  a.expA = p->exp_a;
+  a.expB = p->exp_b;
+  a.need = p->limb_need;
+  a.flag = p->d_flag;
+  a.shift = 6;
+  while (((int64_t)1 << (a.shift - 6)) < p->L) ++a.shift;
+  stark_status st = to_status(launch_leaf_limb(a, &p->tmLA, &p->tmLB, &p->tmSA, &p->tmSB, f64, p->num_sms, s));
+  if (cudaEvent_t* ev = plan_timing_events(p)) {
+    cudaEventRecord(ev[3], s);  // the leaf products end
+    p->timing_leaf_marked = true;
+  }
+  if (st == STARK_OK && stored && p->depth > 0)
+    st = to_status(launch_combine_limb(p->limb_m, p->depth, p->L, core_side(p), C, p->n, p->X, f64, s));
+  if (st != STARK_OK || !f64) return st;
+  st = to_status(launch_gated_clear(C, core_side(p), p->n, p->d_flag, p->num_sms, s));
+  for (int side = 0; side < 2 && st == STARK_OK; ++side) {
+    DivideArgs d{side ? B : A, core_side(p), p->npad, p->L, side ? p->Y : p->X, nullptr, p->d_err, -1, p->n};
+    d.gate = p->d_flag;
+    st = to_status(launch_divide(d, p->depth, side, kInF64, kOutPlain, s));
+  }
+  if (st != STARK_OK) return st;
+  LeafCcArgs c{};
+  c.P = (int32_t)p->P;
+  c.L = (int32_t)p->L;
+  c.leaf_begin = (int32_t)lb;
+  c.leaf_end = (int32_t)le;
+  c.X = p->X;
+  c.Y = p->Y;
+  c.ctab = p->d_ctab;
+  c.ccount = p->d_ccount;
+  c.maxT = p->maxT;
+  c.C = C;
+  c.ldc = p->n;
+  c.n = core_side(p);
+  c.gate = p->d_flag;
+  return to_status(launch_leaf_f64(c, s));
+}
+
 // The peeled edge of a product with n = m + r (Ct: C or its staging copy,
 // row stride ldc): the rank-r update of the core and the two edge strips,
 //   C[:m, :m] += A[:m, m:] B[m:, :m],  C[:m, m:] = A[:m, :] B[:, m:],
@@ -1197,6 +1429,11 @@ stark_status plan_run_accumulate(stark_plan_s* p, const void* A, const void* B, 
       cudaEventRecord(ev[3], s);
       p->timing_leaf_marked = true;
     }
+  } else if (!p->dfs && plan_limbs(p)) {
+    st = plan_limb_divide(p, A, B, s);
+    if (st != STARK_OK) return st;
+    if (ev) cudaEventRecord(ev[2], s);
+    st = plan_limb_leaves(p, A, B, C, lb, le, s);
   } else if (!p->dfs) {
     st = plan_divide_top(p, A, B, s, -1, 0, 0);
     if (st != STARK_OK) return st;
@@ -1228,7 +1465,8 @@ stark_status plan_run_accumulate(stark_plan_s* p, const void* A, const void* B, 
   // staging copy into C
   const bool staged = p->is_tc && !plan_stored(p, lb, le) && plan_uses_cstage(p, C);
   if (st == STARK_OK && p->peel > 0 && lb == 0)
-    st = plan_border(p, A, B, staged ? p->cstage : C, staged ? staged_ld(p->n) : p->n, plan_stored(p, lb, le), s);
+    st = plan_border(p, A, B, staged ? p->cstage : C, staged ? staged_ld(p->n) : p->n,
+                     plan_deterministic(p, lb, le) || plan_sib(p, lb, le), s);
   if (st == STARK_OK && staged) st = plan_copy_cstage(p, C, s);
   if (ev && !p->timing_leaf_marked) cudaEventRecord(ev[3], s);  // depth first: one interleaved phase
   if (ev) cudaEventRecord(ev[4], s);

@@ -77,6 +77,22 @@ struct stark_plan_s {
   bool int_tc = false;
   int int_bn = 128;
   CUtensorMap tmAi, tmBi;
+  // I64 and F64 leaves as digit products on the tensor cores (leaf_limb.cu):
+  // breadth first, leaf sides >= 128; X and Y then hold 16 bytes per element
+  // (eight fp16 digit planes per leaf)
+  bool limb_ok = false;    // the plan may take the limb path
+  int64_t op_elem = 0;     // bytes per operand element that X and Y were allocated with
+  CUtensorMap tmLA, tmLB, tmSA, tmSB;
+  void* limb_m = nullptr;    // [P][L][L] stored products, 8 bytes each (depth >= 1)
+  void* limb_aux = nullptr;  // F64: the arrays below, in one allocation
+  double* max_a = nullptr;   // [2^depth][npad] block maxima of A's rows
+  double* max_b = nullptr;   // and of B's columns
+  int32_t* exp_a = nullptr;  // [P][L] exponents of the leaf operands' rows
+  int32_t* exp_b = nullptr;  // and columns
+  void* mag_a = nullptr;     // [P][L][128] magnitudes of the leading digits
+  void* mag_b = nullptr;     // [P][128][L]
+  float* limb_need = nullptr;  // [P] magnitude sums that prove a leaf's elements
+  int* d_flag = nullptr;     // set when the product must be redone on the CUDA cores
   CUtensorMap tmA;
   CUtensorMap tmB;
   // end-to-end staging (stark_mul_host / _async), allocated on first use:
@@ -115,7 +131,13 @@ namespace stark {
 // dfs: allocate the workspace for the depth-first traversal over that many
 // top levels (one subtree's operands) from the start; traversal_supported
 // must hold for it.
-stark_status plan_init(stark_plan_s* p, int64_t n, int depth, stark_dtype dt, bool peel = false, int dfs = 0);
+// lean: F64 and I64 plans keep to 8 bytes per operand element and the CUDA
+// cores (the server counts these bytes against its budget).
+stark_status plan_init(stark_plan_s* p, int64_t n, int depth, stark_dtype dt, bool peel = false, int dfs = 0,
+                       bool lean = false);
+// Depth of a plan made with depth -1 for F64 and I64 (the server, whose plans
+// are lean, uses choose_depth).
+int choose_plan_depth(int64_t n, stark_dtype dt);
 // Whether the depth-first traversal over `levels` top levels exists for this
 // depth and dtype (subtree loaders cover depth <= 3; two levels only for the
 // split dtypes).  0 (breadth first) always does.

@@ -217,7 +217,7 @@ stark_plan_s* acquire_workspace(stark_server_s* s, const Request& r, stark_statu
     *err = STARK_ENOMEM;
     return nullptr;
   }
-  stark_status st = plan_init(p, npad, d, r.dt, false, levels);  // sized for the whole bucket
+  stark_status st = plan_init(p, npad, d, r.dt, false, levels, true);  // sized for the whole bucket
   if (st == STARK_OK && stage) st = plan_ensure_cstage(p);
   if (st != STARK_OK) {
     plan_release(p);

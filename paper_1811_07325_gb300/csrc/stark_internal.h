@@ -60,7 +60,8 @@ inline bool is_split(stark_dtype dt) {
 inline bool half_split(stark_dtype dt) { return dt == STARK_F32_SPLIT_BF16 || dt == STARK_F32_SPLIT_FP16; }
 
 // ------------------------------------------------------------------ launches
-enum OutMode { kOutSplitBf16 = 0, kOutSplitTf32 = 1, kOutPlain = 2, kOutBf16Exact = 3, kOutSplitFp16 = 4 };
+enum OutMode { kOutSplitBf16 = 0, kOutSplitTf32 = 1, kOutPlain = 2, kOutBf16Exact = 3, kOutSplitFp16 = 4,
+               kOutLimbs = 5 };
 enum InType { kInF32 = 0, kInF64 = 1, kInI64 = 2 };
 
 struct DivideArgs {
@@ -78,6 +79,12 @@ struct DivideArgs {
                       // full padded side >> top_levels)
   int64_t ld;         // row stride of X in elements (>= n)
   int top_levels;     // levels above the subtree (1, or 2 for the split dtypes) when top >= 0
+  const int* gate;    // not null: the launch does nothing unless *gate != 0
+  // kOutLimbs, F64 input: exponents [leaf][L] of the operand's rows (side 0)
+  // or columns (side 1), and the digit-magnitude planes of the first 128 of K
+  // ([leaf][L][128] for side 0, [leaf][128][L] for side 1)
+  const int32_t* exps;
+  void* mags;
 };
 
 // Divide phase for one operand: writes the 7^depth leaf operand sums as
@@ -90,6 +97,28 @@ cudaError_t launch_divide_top(const DivideArgs& a, int depth, int side, InType i
 // needs L % 128 == 0 (divide_staged_fits).  Same planes as launch_divide.
 bool divide_staged_fits(int64_t L);
 cudaError_t launch_divide_staged(const DivideArgs& a, int side, OutMode out, cudaStream_t s);
+// Both operands' digit planes for the limb leaves (kOutLimbs, breadth first,
+// any depth 0..4) in one launch; in: kInI64 or kInF64.
+cudaError_t launch_divide_limbs(const DivideArgs& a, const DivideArgs& b, int depth, InType in, cudaStream_t s);
+
+// F64 limb operands: bounds of the rows of every A leaf operand and the
+// columns of every B leaf operand (limb_bounds.cu).
+struct LimbBoundsArgs {
+  const double* A;
+  const double* B;
+  int64_t n, ld;      // side read, row stride
+  int64_t npad, L;
+  int depth;
+  double* max_a;      // [2^depth column blocks][npad]: row maxima of |A|
+  double* max_b;      // [2^depth row blocks][npad]: column maxima of |B|
+  int32_t* expA;      // [7^depth][L]
+  int32_t* expB;
+  int* flag;          // cleared, then set for infinities, NaN and exponents outside +-400
+};
+cudaError_t launch_limb_bounds(const LimbBoundsArgs& a, cudaStream_t s);
+// C = 0 where *gate != 0 (n x n elements of 8 bytes, row stride ld).
+cudaError_t launch_gated_clear(void* C, int64_t n, int64_t ld, const int* gate, int num_sms, cudaStream_t s);
+
 // C (+)= A B on sub-blocks (M x K times K x N, row strides lda, ldb, ldc in
 // elements) on the CUDA cores: the edges of a peeled product.  Element type
 // float (fp32 accumulate), double or int64 (wrapping); accumulate = 0
@@ -114,6 +143,9 @@ cudaError_t launch_border(const BorderArgs& a, InType t, int num_sms, cudaStream
 cudaError_t launch_combine(const float* M, int depth, int64_t L, int64_t npad, int64_t n, float* C, int64_t ldc,
                            cudaStream_t s);
 bool make_tmap_mplanes(CUtensorMap* m, void* base, int64_t L, int64_t planes);
+// [planes][rows][cols] of 16-bit elements; boxes of 64 or 32 columns (128- or 64-byte swizzle).
+bool make_tmap_half3(CUtensorMap* m, void* base, int64_t cols, int64_t rows, int64_t planes, int box_cols, int box_rows,
+                     int box_planes);
 // In-place transpose of `count` square L x L fp32 planes.
 cudaError_t launch_transpose_planes(float* planes, int64_t L, int64_t count, cudaStream_t s);
 
@@ -203,9 +235,43 @@ struct LeafCcArgs {
   int32_t maxT;
   void* C;
   int64_t ldc, n;
+  const int* gate;  // not null: the launch does nothing unless *gate != 0
 };
 cudaError_t launch_leaf_f64(const LeafCcArgs& a, cudaStream_t s);
 cudaError_t launch_leaf_i64(const LeafCcArgs& a, cudaStream_t s);
+
+// Leaves of the I64 and F64 dtypes as digit products on the tensor cores
+// (leaf_limb.cu): operands in [leaf][8] planes of L x L fp16 digits, leaf side
+// L >= 128 a multiple of 64.
+constexpr int32_t kLimbZeroRow = INT32_MIN;  // exponent of an operand row (column) that is zero
+constexpr int kLimbCheckK = 128;             // K of the F64 magnitude check's planes
+struct LeafLimbArgs {
+  int32_t L, leaf_begin, leaf_end;
+  const CTarget* ctab;
+  const int32_t* ccount;
+  int32_t maxT;
+  void* C;  // double or int64, accumulated into; with `store` overwritten
+  int64_t ldc, n;
+  // not null: products are stored, leaf l at store + l L^2 (row pitch L), or,
+  // at depth 0, straight into C (store == C)
+  void* store;
+  int* err;
+  uint64_t timeout_ns;
+  // F64 only
+  const int32_t* expA;  // [leaf][L]: exponent e of a row of A, |x| <= 2^e (kLimbZeroRow: all zero)
+  const int32_t* expB;  // [leaf][L]: the same of a column of B
+  const float* need;    // [leaf]: digit-magnitude sum that proves an element (limb_check_sum)
+  int32_t shift;        // the running sums' unit, 2^shift of 256^7: log2(L) rounded up, plus 6
+  int* flag;            // set to 1 when an element's accuracy is not proven
+};
+cudaError_t launch_leaf_limb(const LeafLimbArgs& a, const CUtensorMap* tmA, const CUtensorMap* tmB,
+                             const CUtensorMap* tmSA, const CUtensorMap* tmSB, bool f64, int num_sms,
+                             cudaStream_t s);
+
+// Ordered combine of the stored limb products M [7^depth][L][L] into C (depth
+// 1..4); tmp: 7^(depth - 2) (4 L)^2 elements for depths 3 and 4.
+cudaError_t launch_combine_limb(const void* M, int depth, int64_t L, int64_t n, void* C, int64_t ldc, void* tmp,
+                                bool f64, cudaStream_t s);
 
 cudaError_t launch_wait_selftest(int* err, uint64_t timeout_ns, cudaStream_t s);
 

@@ -338,7 +338,8 @@ stark_status stark_batch_mul(stark_batch_t b, const void* const* A, const void* 
       const bool staged = plan_uses_cstage(b->plans[k], Cuser);
       g.C = static_cast<float*>(staged ? b->plans[k]->cstage : Cuser);
       g.ldc = staged ? staged_ld(g.n) : g.n;
-      g.use_tma_c = make_tmap_c(&g.tmC, g.C, g.n, g.ldc) ? 1 : 0;
+      // (one leaf: each element of C is stored once, not added into a cleared C)
+      g.use_tma_c = make_tmap_c(&g.tmC, g.C, g.n, g.ldc) ? (b->plans[k]->depth == 0 ? 2 : 1) : 0;
     }
     if (cudaMemcpy(b->d_desc, b->host_desc.data(), sizeof(GroupDesc) * count, cudaMemcpyHostToDevice) !=
         cudaSuccess)
@@ -360,10 +361,8 @@ stark_status stark_batch_mul(stark_batch_t b, const void* const* A, const void* 
       stark_plan_s* p = b->plans[k];
       const GroupDesc& g = b->host_desc[k];
       cudaStream_t sk = b->side[k % F];
-      if (cudaMemsetAsync(g.C, 0, (size_t)p->n * g.ldc * sizeof(float), sk) != cudaSuccess)
-        st = STARK_ECUDA;
-      else
-        st = plan_divide(p, ptrs[3 * k], ptrs[3 * k + 1], sk);
+      st = plan_divide_clear(p, ptrs[3 * k], ptrs[3 * k + 1], g.use_tma_c == 2 ? nullptr : g.C,
+                             (size_t)p->n * g.ldc * sizeof(float), sk);
     }
     for (int i = 0; i < F; ++i)  // join (also after an error, so the capture can end)
       if (cudaEventRecord(b->join_ev[i], b->side[i]) != cudaSuccess ||

@@ -27,13 +27,18 @@ namespace {
 
 template <typename Tin, int OUT, int SIDE>
 cudaError_t by_depth(const DivideArgs& a, int depth, cudaStream_t st) {
-  switch (depth) {
-    case 0: return launch_one<Tin, OUT, 0, SIDE, 0>(a, st);
-    case 1: return launch_one<Tin, OUT, 1, SIDE, 0>(a, st);
-    case 2: return launch_one<Tin, OUT, 2, SIDE, 0>(a, st);
-    case 3: return launch_one<Tin, OUT, 3, SIDE, 0>(a, st);
-    case 4: return launch_one<Tin, OUT, 4, SIDE, 0>(a, st);
-    default: return cudaErrorInvalidValue;
+  if constexpr (std::is_same_v<Tin, float>) {
+    // split dtypes: depths 0..2 in divide_pair.cu, 3 in divide_staged.cu
+    return depth == 4 ? launch_one<Tin, OUT, 4, SIDE, 0>(a, st) : cudaErrorInvalidValue;
+  } else {
+    switch (depth) {
+      case 0: return launch_one<Tin, OUT, 0, SIDE, 0>(a, st);
+      case 1: return launch_one<Tin, OUT, 1, SIDE, 0>(a, st);
+      case 2: return launch_one<Tin, OUT, 2, SIDE, 0>(a, st);
+      case 3: return launch_one<Tin, OUT, 3, SIDE, 0>(a, st);
+      case 4: return launch_one<Tin, OUT, 4, SIDE, 0>(a, st);
+      default: return cudaErrorInvalidValue;
+    }
   }
 }
 
@@ -52,8 +57,8 @@ cudaError_t launch_divide(const DivideArgs& a, int depth, int side, InType in, O
   if (in == kInI64 && out == kOutPlain)
     return side == 0 ? by_depth<int64_t, kOutPlain, 0>(a, depth, st) : by_depth<int64_t, kOutPlain, 1>(a, depth, st);
   if (in == kInI64 && out == kOutBf16Exact)
-    return side == 0 ? by_depth<int64_t, kOutBf16Exact, 0>(a, depth, st)
-                     : by_depth<int64_t, kOutBf16Exact, 1>(a, depth, st);
+    return side == 0 ? by_depth<SmallI64, kOutBf16Exact, 0>(a, depth, st)
+                     : by_depth<SmallI64, kOutBf16Exact, 1>(a, depth, st);
   return cudaErrorInvalidValue;
 }
 

@@ -25,6 +25,27 @@ struct AccOf<int64_t> {
   using type = unsigned long long;  // wraps modulo 2^64
 };
 
+// An int64 input of the exact bf16 operands (|sums| <= 256): sums in 32 bits,
+// so that a thread can hold four columns.  Inputs are clamped to 2^20, which
+// changes no verdict: were every leaf sum of a larger input within 256, the
+// quadrants that stand alone in a product (11 and 22) would be, and with them
+// the others within 512 a level.
+struct SmallI64 {
+  long long v;
+  __host__ __device__ explicit operator int() const {
+    return (int)(v > (1 << 20) ? (1 << 20) : v < -(1 << 20) ? -(1 << 20) : v);
+  }
+};
+template <>
+struct AccOf<SmallI64> {
+  using type = int;
+};
+__device__ __forceinline__ SmallI64 load_one(const SmallI64* p) { return SmallI64{__ldcs(&p->v)}; }
+template <typename T>
+__device__ __forceinline__ T load_one(const T* p) {
+  return __ldcs(p);
+}
+
 // The two-term sums of Alg. 1 for product m (0..6 = M1..M7), quadrant values
 // from g(q), q = 0:11, 1:12, 2:21, 3:22.
 template <int SIDE, typename V, class Get>
@@ -154,7 +175,7 @@ struct Emitter {
       bool bad = false;
 #pragma unroll
       for (int e = 0; e < VEC; ++e) {
-        const long long v = (long long)x.v[e];
+        const int v = (int)x.v[e];
         bad |= (v > 256 || v < -256);
         h[e] = __float2bfloat16_rn((float)v);
       }
@@ -263,19 +284,22 @@ struct Loader {
     Vec<Acc, VEC> r;
     if (row < n && col + VEC <= n && vec_ok) {
       const Tin* p = X + row * ld + col;
-      if constexpr (sizeof(Tin) * VEC == 16) {
-        const int4 raw = __ldcs(reinterpret_cast<const int4*>(p));
-        const Tin* t = reinterpret_cast<const Tin*>(&raw);
+      if constexpr (sizeof(Tin) * VEC % 16 == 0) {
+        constexpr int W = (int)sizeof(Tin) * VEC / 16;
+        int4 raw[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) raw[w] = __ldcs(reinterpret_cast<const int4*>(p) + w);
+        const Tin* t = reinterpret_cast<const Tin*>(raw);
 #pragma unroll
         for (int e = 0; e < VEC; ++e) r.v[e] = (Acc)t[e];
       } else {
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) r.v[e] = (Acc)__ldcs(p + e);
+        for (int e = 0; e < VEC; ++e) r.v[e] = (Acc)load_one(p + e);
       }
     } else {
 #pragma unroll
       for (int e = 0; e < VEC; ++e)
-        r.v[e] = (row < n && col + e < n) ? (Acc)__ldcs(X + row * ld + col + e) : Acc(0);
+        r.v[e] = (row < n && col + e < n) ? (Acc)load_one(X + row * ld + col + e) : Acc(0);
     }
     return r;
   }
@@ -454,16 +478,17 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
 
 template <typename Tin, int OUT, int D, int SIDE, int VEC, int K>
 __global__ void __launch_bounds__(256, 2) divide_kernel(DivideArgs a, int vec_ok) {
-  if (a.gate && *(volatile const int*)a.gate == 0) return;
   divide_body<Tin, OUT, D, SIDE, VEC, K>(a, vec_ok);
 }
 
 template <typename Tin, int OUT, int D, int SIDE, int K>
 cudaError_t launch_one(const DivideArgs& a, cudaStream_t st) {
-  constexpr int VEC = 16 / (int)sizeof(Tin);  // one 16-byte load per quadrant
+  // one 16-byte load per quadrant; the small integers take two, for 8-byte
+  // stores (51 us an operand with 4-byte ones at n = 4096, depth 1)
+  constexpr int VEC = (std::is_same_v<Tin, SmallI64> ? 32 : 16) / (int)sizeof(Tin);
   if (a.L % VEC != 0) return cudaErrorInvalidValue;
   if (a.ld < a.n) return cudaErrorInvalidValue;
-  const int vec_ok = (a.ld % VEC == 0) && ((reinterpret_cast<uintptr_t>(a.X) & 15) == 0);
+  const int vec_ok = (a.ld % (16 / (int)sizeof(Tin)) == 0) && ((reinterpret_cast<uintptr_t>(a.X) & 15) == 0);
   const int64_t threads = a.L * (a.L / VEC);
   const int64_t blocks = (threads + 255) / 256;
   if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;

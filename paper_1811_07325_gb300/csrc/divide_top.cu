@@ -50,8 +50,8 @@ cudaError_t launch_divide_top(const DivideArgs& a, int depth, int side, InType i
     return side == 0 ? by_depth_top<int64_t, kOutPlain, 0>(a, depth, st)
                      : by_depth_top<int64_t, kOutPlain, 1>(a, depth, st);
   if (in == kInI64 && out == kOutBf16Exact)
-    return side == 0 ? by_depth_top<int64_t, kOutBf16Exact, 0>(a, depth, st)
-                     : by_depth_top<int64_t, kOutBf16Exact, 1>(a, depth, st);
+    return side == 0 ? by_depth_top<SmallI64, kOutBf16Exact, 0>(a, depth, st)
+                     : by_depth_top<SmallI64, kOutBf16Exact, 1>(a, depth, st);
   return cudaErrorInvalidValue;
 }
 

@@ -15,6 +15,7 @@ struct ItemInfo {
   const CUtensorMap* tB;
   const CUtensorMap* tC;
   int leaf, P, m0, n0, kblocks;
+  int kb0;     // first K block (a slice of a split K range)
   const CTarget* tg;
   int nt;
   float* C;
@@ -60,6 +61,7 @@ __device__ __forceinline__ ItemInfo decode_sib(int item, const LeafTcArgs& p, co
   it.m0 = ((tile / tiles_n) * 2 + (int)rank) * kBM;
   it.n0 = (tile % tiles_n) * BN;
   it.kblocks = p.L / BK;
+  it.kb0 = 0;
   it.tg = nullptr;
   it.nt = 0;
   it.C = p.C;
@@ -120,6 +122,7 @@ __device__ __forceinline__ ItemInfo decode_item(int item, const LeafTcArgs& p, c
     it.m0 = PAIR ? (((rem % per_leaf) / tiles_n) * 2 + (int)rank) * kBM : ((rem % per_leaf) / tiles_n) * kBM;
     it.n0 = ((rem % per_leaf) % tiles_n) * BN;
     it.kblocks = L / BK;
+    it.kb0 = 0;
     it.tg = g->ctab + (int64_t)it.leaf * g->maxT;
     it.nt = g->ccount[it.leaf];
     it.C = g->C;
@@ -133,6 +136,13 @@ __device__ __forceinline__ ItemInfo decode_item(int item, const LeafTcArgs& p, c
     const int tiles_n = p.L / BN;
     const int tiles_m = p.L / kBM / (PAIR ? 2 : 1);
     const int per_leaf = tiles_m * tiles_n;
+    it.kblocks = p.L / BK;
+    it.kb0 = 0;
+    if (p.ksplit > 1) {  // (a power of two that divides the K blocks)
+      it.kblocks /= p.ksplit;
+      it.kb0 = item % p.ksplit * it.kblocks;
+      item /= p.ksplit;
+    }
     const int rem = item % per_leaf;
     int row, col;
     if (p.band > 0 && p.band < tiles_n && tiles_n % p.band == 0) {
@@ -153,7 +163,6 @@ __device__ __forceinline__ ItemInfo decode_item(int item, const LeafTcArgs& p, c
     it.P = p.P;
     it.m0 = PAIR ? (row * 2 + (int)rank) * kBM : row * kBM;
     it.n0 = col * BN;
-    it.kblocks = p.L / BK;
     it.tg = p.ctab + (int64_t)it.leaf * p.maxT;
     it.nt = p.ccount[it.leaf];
     it.C = p.C;
@@ -195,7 +204,7 @@ __device__ __forceinline__ void epilogue_item(const ItemInfo& it, const LeafTcAr
     uint32_t r[32];
     tmem_ld_32x32b_x32(tmem_base + ((uint32_t)(quarter * 32) << 16) + acc_col + (uint32_t)(chunk * 32), r);
     tmem_ld_wait();
-    if constexpr (INT1) {
+    if (INT1 && !p.store_m) {
       // exact integers held in fp32: signed 64-bit adds into C (wrap mod
       // 2^64).  A whole, 16-byte-aligned row segment goes as one bulk
       // add-reduction of 256 bytes from this thread's slot of `ebuf`
@@ -286,9 +295,13 @@ __device__ __forceinline__ void epilogue_item(const ItemInfo& it, const LeafTcAr
     } else if (p.store_m) {
       // unfused, deterministic combine: this leaf's tile goes to its M
       // plane (tmC maps the M planes here); the combine kernel adds later
-      if (lane == 0) bulk_wait_group_read<0>();
+      // (the two boxes in turn: the one before last has been read)
+      const uint32_t box = ebuf + (uint32_t)(chunk & 1) * 4096u;
+      if (lane == 0) {
+        if (chunk == 0) bulk_wait_group_read<0>(); else bulk_wait_group_read<1>();
+      }
       __syncwarp();
-      const uint32_t row_addr = ebuf + (uint32_t)lane * 128u;
+      const uint32_t row_addr = box + (uint32_t)lane * 128u;
 #pragma unroll
       for (int c = 0; c < 8; ++c) {
         const uint32_t addr = row_addr + ((uint32_t)(c ^ (lane & 7)) << 4);
@@ -301,16 +314,22 @@ __device__ __forceinline__ void epilogue_item(const ItemInfo& it, const LeafTcAr
       if (lane == 0) {
         // the planes are read back only by the combine pass, after the whole
         // launch: evict-first keeps them from displacing operand panels in L2
-        tma_store_3d_hint(it.tC, n0 + chunk * 32, m0 + quarter * 32, it.leaf - p.leaf_begin, ebuf, pol_c);
+        tma_store_3d_hint(it.tC, n0 + chunk * 32, m0 + quarter * 32, it.leaf - p.leaf_begin, box, pol_c);
         bulk_commit_group();
       }
     } else if (it.use_tma_c) {
-      if (lane == 0) bulk_wait_group_read<0>();  // the previous boxes have been read
+      // a tile of one sign takes the two boxes in turn, else they hold the
+      // tile and its negation
+      const bool turn = !has_neg;
+      const uint32_t pbox = ebuf + (turn ? (uint32_t)(chunk & 1) * 4096u : 0u);
+      if (lane == 0) {
+        if (turn && chunk > 0) bulk_wait_group_read<1>(); else bulk_wait_group_read<0>();
+      }
       __syncwarp();
 #pragma unroll
       for (int sg = 0; sg < 2; ++sg) {
         if (sg == 0 ? !has_pos : !has_neg) continue;
-        const uint32_t row_addr = ebuf + (uint32_t)sg * 4096u + (uint32_t)lane * 128u;
+        const uint32_t row_addr = (sg == 0 ? pbox : ebuf + 4096u) + (uint32_t)lane * 128u;
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
           float4 v = make_float4(__uint_as_float(r[4 * c]), __uint_as_float(r[4 * c + 1]),
@@ -330,7 +349,10 @@ __device__ __forceinline__ void epilogue_item(const ItemInfo& it, const LeafTcAr
           const int64_t y = (int64_t)c.row_off + m0 + quarter * 32;
           const int64_t x = (int64_t)c.col_off + n0 + chunk * 32;
           if (y >= it.n || x >= it.n) continue;
-          tma_reduce_add_2d(it.tC, (int32_t)x, (int32_t)y, ebuf + (c.sign > 0 ? 0u : 4096u), pol_c);
+          if (it.use_tma_c == 2)
+            tma_store_2d_hint(it.tC, (int32_t)x, (int32_t)y, pbox, pol_c);
+          else
+            tma_reduce_add_2d(it.tC, (int32_t)x, (int32_t)y, c.sign > 0 ? pbox : ebuf + 4096u, pol_c);
         }
         bulk_commit_group();
       }
@@ -413,7 +435,10 @@ __device__ __forceinline__ void epilogue_box_regs(const ItemInfo& it, const Leaf
           const int64_t y = (int64_t)c.row_off + m0 + quarter * 32;
           const int64_t x = (int64_t)c.col_off + n0 + col0;
           if (y >= it.n || x >= it.n) continue;
-          tma_reduce_add_2d(it.tC, (int32_t)x, (int32_t)y, ebuf, pol_c);
+          if (it.use_tma_c == 2)
+            tma_store_2d_hint(it.tC, (int32_t)x, (int32_t)y, ebuf, pol_c);
+          else
+            tma_reduce_add_2d(it.tC, (int32_t)x, (int32_t)y, ebuf, pol_c);
         }
         bulk_commit_group();
       }
@@ -453,7 +478,9 @@ cudaError_t launch_cta_pairs(Kern kern, int threads, int smem, int64_t items, in
                              const CUtensorMap& tmA, const CUtensorMap& tmB, const CUtensorMap& tmC,
                              const LeafTcArgs& a) {
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
@@ -462,7 +489,7 @@ cudaError_t launch_cta_pairs(Kern kern, int threads, int smem, int64_t items, in
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 1;  // (occupancy query)
   int clusters = num_sms / 2;
   cfg.gridDim = dim3((unsigned)(2 * clusters), 1, 1);
   int active = 0;
@@ -471,6 +498,7 @@ cudaError_t launch_cta_pairs(Kern kern, int threads, int smem, int64_t items, in
   cudaGetLastError();
   if (items < clusters) clusters = (int)items;
   cfg.gridDim = dim3((unsigned)(2 * clusters), 1, 1);
+  cfg.numAttrs = a.pdl ? 2 : 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, kern, tmA, tmB, tmC, a);
   count_launch();
   return e != cudaSuccess ? e : cudaGetLastError();

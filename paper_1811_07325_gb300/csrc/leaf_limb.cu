@@ -72,7 +72,7 @@ constexpr int kQuadBytes = 32768;                  // four digit planes: 128 row
 constexpr int kQuads = 6;
 constexpr int kEpiStride = 72;                     // bytes per staged row of 8 results: 64, and 8 so that the
                                                    // rows start in different banks
-constexpr int kEpiBytes = 8 * 32 * kEpiStride;
+constexpr int kEpiBytes = 8 * (32 * kEpiStride + 256);  // and the exponents of each warp's 64 columns
 constexpr int kBarBytes = 8 * (2 * kQuads + 8) + 16;
 constexpr int kSmemLimb = kQuads * kQuadBytes + kEpiBytes + 1024 + kBarBytes;
 static_assert(kSmemLimb <= 232448, "shared memory per CTA");
@@ -82,19 +82,17 @@ __device__ __forceinline__ long long add_high(long long acc, int v) {
   return (long long)(((unsigned long long)hi << 32) | (uint32_t)acc);
 }
 
-// v * 2^e rounded to nearest even, from integer operations (the FP64 pipe
-// does two operations a clock); |result| stays in the normal range.
+// v * 2^e rounded to nearest (ties away), from integer operations (the FP64
+// pipe does two operations a clock); |result| stays in the normal range.
 __device__ __forceinline__ unsigned long long scaled_double_bits(long long v, int e) {
-  if (v == 0) return 0ull;
-  const unsigned long long sign = v < 0 ? 0x8000000000000000ull : 0ull;
-  unsigned long long u = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  const long long sign = v >> 63;
+  unsigned long long u = (unsigned long long)((v ^ sign) - sign);
   const int lz = __clzll((long long)u);
-  u <<= lz;  // bit 63 set
-  const unsigned long long rest = u & 2047ull;
-  unsigned long long m = u >> 11;  // 53 bits
-  m += (rest > 1024ull || (rest == 1024ull && (m & 1ull))) ? 1ull : 0ull;
-  // m == 2^53 carries into the exponent by the addition
-  return sign | (((unsigned long long)(e + 63 - lz + 1022) << 52) + m);
+  u <<= lz & 63;  // bit 63 set
+  // 53 bits and the rounding; a carry to 2^53 goes into the exponent
+  const unsigned long long m = (u >> 11) + ((u >> 10) & 1ull);
+  const unsigned long long bits = ((unsigned long long)(unsigned)(e + 1085 - lz) << 52) + m;
+  return v == 0 ? 0ull : bits | ((unsigned long long)sign & 0x8000000000000000ull);
 }
 
 template <bool F64>
@@ -379,7 +377,8 @@ __global__ void __launch_bounds__(kThreadsL, 1)
     const int quarter = warp & 3;
     const int half = (warp - 4) >> 2;
     const uint32_t lane_base = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * 64);
-    const uint32_t ebuf = epi_base + (uint32_t)(warp - 4) * (32 * kEpiStride);
+    const uint32_t ebuf = epi_base + (uint32_t)(warp - 4) * (32 * kEpiStride + 256);
+    const uint32_t fbuf = ebuf + 32 * kEpiStride;
     uint32_t acc_phase = 0;
     bool ok = true;
     long long sum[64];
@@ -432,11 +431,21 @@ __global__ void __launch_bounds__(kThreadsL, 1)
       const int row0 = tile / tiles * 128 + quarter * 32, row = row0 + lane;  // in the leaf plane
       const int col0 = tile % tiles * 128 + half * 64;
       int ea = 0;
-      const int32_t* fb = nullptr;
+      auto fexp = [&](int c) {  // exponent of column col0 + c
+        int f;
+        asm volatile("ld.shared.s32 %0, [%1];" : "=r"(f) : "r"(fbuf + 4u * (uint32_t)c));
+        return f;
+      };
       if (F64) {
-        const int32_t* eap = p.expA + (int64_t)leaf * p.L;
-        fb = p.expB + (int64_t)leaf * p.L;
-        ea = row < p.L ? eap[row] : kLimbZeroRow;
+        const int32_t* fb = p.expB + (int64_t)leaf * p.L;
+        ea = row < p.L ? p.expA[(int64_t)leaf * p.L + row] : kLimbZeroRow;
+        __syncwarp();  // (the previous tile's exponents have been read)
+#pragma unroll
+        for (int h = 0; h < 64; h += 32) {
+          const int f = col0 + h + lane < p.L ? fb[col0 + h + lane] : kLimbZeroRow;
+          asm volatile("st.shared.s32 [%0], %1;" ::"r"(fbuf + 4u * (uint32_t)(h + lane)), "r"(f) : "memory");
+        }
+        __syncwarp();
         const float need = p.need[leaf];  // the magnitude check of every element that can be non-zero
         if (!wait_acc(3)) break;
         bool bad = false;
@@ -447,9 +456,7 @@ __global__ void __launch_bounds__(kThreadsL, 1)
           tmem_ld_wait();
 #pragma unroll
           for (int e = 0; e < 16; ++e) {
-            const int c = col0 + j * 16 + e;
-            if (!(__uint_as_float(r[e]) >= need) && ea != kLimbZeroRow && c < p.L && fb[c] != kLimbZeroRow)
-              bad = true;
+            if (!(__uint_as_float(r[e]) >= need) && ea != kLimbZeroRow && fexp(j * 16 + e) != kLimbZeroRow) bad = true;
           }
         }
         free_acc(3);
@@ -473,15 +480,9 @@ __global__ void __launch_bounds__(kThreadsL, 1)
         unsigned long long v[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
-          if (F64) {
-            const int c = col0 + j * 8 + e;
-            const int f = c < p.L ? fb[c] : kLimbZeroRow;
-            v[e] = (ea == kLimbZeroRow || f == kLimbZeroRow)
-                       ? 0ull
-                       : scaled_double_bits(sum[j * 8 + e], ea + f + p.shift - 68);
-          } else {
-            v[e] = (unsigned long long)sum[j * 8 + e];
-          }
+          // (a zero row or column has a zero sum, whatever its exponent says)
+          v[e] = F64 ? scaled_double_bits(sum[j * 8 + e], ea + fexp(j * 8 + e) + p.shift - 68)
+                     : (unsigned long long)sum[j * 8 + e];
         }
         // turned in shared memory so that a warp writes four row pieces of 64
         // bytes at a time (per-row bulk reductions of 64 bytes from the staged

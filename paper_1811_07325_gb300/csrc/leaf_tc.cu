@@ -94,7 +94,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   const uint32_t cta_rank = 0u;
   const int unit = (int)blockIdx.x;
   const int units = (int)gridDim.x;
-  const int num_items = GROUPED ? p.total_items : (p.leaf_end - p.leaf_begin) * (p.L / kBM) * (p.L / BN);
+  const int num_items = GROUPED ? p.total_items
+                                : (p.leaf_end - p.leaf_begin) * (p.L / kBM) * (p.L / BN) * (p.ksplit > 1 ? p.ksplit : 1);
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
@@ -109,7 +110,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     if (!GROUPED) {
       prefetch_tmap(&tmA);
       prefetch_tmap(&tmB);
-      if (p.use_tma_c) prefetch_tmap(&tmC);
+      if (p.use_tma_c || p.store_m) prefetch_tmap(&tmC);
     }
   }
   if (warp == 1) {
@@ -120,6 +121,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();  // the operands (and a cleared C) of a divide still running
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
@@ -149,7 +151,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           const uint32_t st = sbase + s * Cfg::STAGE_BYTES;
           mbar_arrive_expect_tx(full_bar(s), Cfg::STAGE_BYTES);
-          const int k0 = kb * Cfg::BK;
+          const int k0 = (it.kb0 + kb) * Cfg::BK;
           tma_load_3d(st, it.tA, k0, m0, leaf, full_bar(s), pol_a);
           if constexpr (!INT1) tma_load_3d(st + Cfg::A_BYTES, it.tA, k0, m0, it.P + leaf, full_bar(s), pol_a);
           if constexpr (Cfg::B_MN) {
@@ -190,7 +192,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool issued = false;
       for (int item = unit; ok && item < num_items; item += units) {
         const int kblocks = GROUPED ? decode_item<BN, Cfg::BK, GROUPED, false>(item, p, &tmA, &tmB, &tmC, cta_rank).kblocks
-                                    : p.L / Cfg::BK;
+                                    : p.L / Cfg::BK / (p.ksplit > 1 ? p.ksplit : 1);
         if (!mbar_wait_bounded(acce_bar(acc), acc_phase ^ 1, p.err, kDevTimeoutAccEmpty, p.timeout_ns)) {
           ok = false;
           break;
@@ -296,7 +298,8 @@ cudaError_t launch_cfg(const LeafTcArgs& a, const CUtensorMap* tmA, const CUtens
     if (!a.groups || a.ngroups <= 0) return cudaErrorInvalidValue;
   } else {
     if (a.L % kBM != 0 || a.L % BN != 0 || a.L % Cfg::BK != 0) return cudaErrorInvalidValue;
-    items = (int64_t)(a.leaf_end - a.leaf_begin) * (a.L / kBM) * (a.L / BN);
+    if (a.ksplit > 1 && (INT1 || a.store_m || (a.L / Cfg::BK) % a.ksplit != 0)) return cudaErrorInvalidValue;
+    items = (int64_t)(a.leaf_end - a.leaf_begin) * (a.L / kBM) * (a.L / BN) * (a.ksplit > 1 ? a.ksplit : 1);
   }
   auto kern = leaf_tc_kernel<BN, STAGES, TF32, GROUPED, RB, INT1, TMN>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
@@ -304,9 +307,19 @@ cudaError_t launch_cfg(const LeafTcArgs& a, const CUtensorMap* tmA, const CUtens
   if (items <= 0) return cudaSuccess;
   if (items > 0x7FFFFFFF) return cudaErrorInvalidValue;
   const int grid = (int)(items < num_sms ? items : num_sms);
-  kern<<<grid, kThreads, Cfg::SMEM, st>>>(*tmA, *tmB, *tmC, a);
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3(kThreads, 1, 1);
+  cfg.dynamicSmemBytes = (size_t)Cfg::SMEM;
+  cfg.stream = st;
+  cfg.attrs = attr;
+  cfg.numAttrs = a.pdl ? 1 : 0;
+  e = cudaLaunchKernelEx(&cfg, kern, *tmA, *tmB, *tmC, a);
   count_launch();
-  return cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 }  // namespace
@@ -332,12 +345,10 @@ cudaError_t launch_leaf_tc(const LeafTcArgs& a, const CUtensorMap* tmA, const CU
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_leaf_tc_int(const LeafTcArgs& a, const CUtensorMap* tmA, const CUtensorMap* tmB, int bn,
-                               int num_sms, cudaStream_t st) {
-  CUtensorMap none;
-  memset(&none, 0, sizeof(none));
-  if (bn == 256) return launch_cfg<256, 4, false, false, 128, true>(a, tmA, tmB, &none, num_sms, st);
-  if (bn == 128) return launch_cfg<128, 6, false, false, 128, true>(a, tmA, tmB, &none, num_sms, st);
+cudaError_t launch_leaf_tc_int(const LeafTcArgs& a, const CUtensorMap* tmA, const CUtensorMap* tmB,
+                               const CUtensorMap* tmC, int bn, int num_sms, cudaStream_t st) {
+  if (bn == 256) return launch_cfg<256, 4, false, false, 128, true>(a, tmA, tmB, tmC, num_sms, st);
+  if (bn == 128) return launch_cfg<128, 6, false, false, 128, true>(a, tmA, tmB, tmC, num_sms, st);
   return cudaErrorInvalidValue;
 }
 

@@ -105,7 +105,7 @@ __global__ void __launch_bounds__(PROMO ? kThreads2P : kThreads2, 1)
   const int units = (int)(gridDim.x >> 1);
   const int num_items = GROUPED ? p.total_items
                         : SIB   ? (int)sib_items(p, Cfg::BN, units)
-                                : (p.leaf_end - p.leaf_begin) * (p.L / (2 * kBM)) * (p.L / Cfg::BN);
+                                : (p.leaf_end - p.leaf_begin) * (p.L / (2 * kBM)) * (p.L / Cfg::BN) * (p.ksplit > 1 ? p.ksplit : 1);
   auto decode = [&](int item) {
     if constexpr (SIB)
       return decode_sib<Cfg::BN, Cfg::BK>(item, p, &tmA, &tmB, &tmC, rank, units);
@@ -137,6 +137,7 @@ __global__ void __launch_bounds__(PROMO ? kThreads2P : kThreads2, 1)
   cluster_sync();  // barriers of both CTAs initialised, TMEM address published
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_wait();  // the operands (and a cleared C) of a divide still running
 
   if (warp == 0) {
     // ------------------------------------------------------------ producer
@@ -165,7 +166,7 @@ __global__ void __launch_bounds__(PROMO ? kThreads2P : kThreads2, 1)
           const uint32_t st = sbase + s * Cfg::STAGE_BYTES;
           const uint32_t fb = mapa_shared(full_bar(s), 0);
           if (leader) mbar_arrive_expect_tx(full_bar(s), 2 * Cfg::STAGE_BYTES);
-          const int k0 = kb * Cfg::BK;
+          const int k0 = (it.kb0 + kb) * Cfg::BK;
           tma_load_3d_cg2(st, it.tA, k0, m0, leaf, fb, pol_a);
           tma_load_3d_cg2(st + Cfg::A_BYTES, it.tA, k0, m0, it.P + leaf, fb, pol_a);
           if constexpr (Cfg::B_MN) {
@@ -286,7 +287,7 @@ __global__ void __launch_bounds__(PROMO ? kThreads2P : kThreads2, 1)
       } else {
         for (int item = unit; ok && item < num_items; item += units) {
           if (SIB && !decode(item).valid) continue;
-          const int kblocks = GROUPED ? decode(item).kblocks : p.L / Cfg::BK;
+          const int kblocks = GROUPED ? decode(item).kblocks : p.L / Cfg::BK / (p.ksplit > 1 ? p.ksplit : 1);
           // both CTAs' epilogues have drained this accumulator
           if (!mbar_wait_bounded_cluster(acce_bar(acc), acc_phase ^ 1, p.err, kDevTimeoutAccEmpty, p.timeout_ns)) {
             ok = false;
@@ -406,7 +407,8 @@ cudaError_t launch2(const LeafTcArgs& a, const CUtensorMap* tmA, const CUtensorM
     if (SIB && (a.leaf_begin % 7 != 0 || (a.leaf_end - a.leaf_begin) % 7 != 0)) return cudaErrorInvalidValue;
     // (sibling-major: the padded item count follows the pairs launched; the
     // kernel derives it, and any count >= the pairs gives the same launch)
-    items = (int64_t)(a.leaf_end - a.leaf_begin) * (a.L / (2 * kBM)) * (a.L / Cfg::BN);
+    if (a.ksplit > 1 && (PROMO || SIB || a.store_m || (a.L / Cfg::BK) % a.ksplit != 0)) return cudaErrorInvalidValue;
+    items = (int64_t)(a.leaf_end - a.leaf_begin) * (a.L / (2 * kBM)) * (a.L / Cfg::BN) * (a.ksplit > 1 ? a.ksplit : 1);
   }
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg::SMEM);
   if (e != cudaSuccess) return e;

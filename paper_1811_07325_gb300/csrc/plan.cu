@@ -750,6 +750,20 @@ stark_status stark_plan_set_input_bound(stark_plan_t p, int64_t max_abs) {
   if (!make_tmap_planes(&p->tmAi, p->X, false, p->L, p->P_ws, 128) ||
       !make_tmap_planes(&p->tmBi, p->Y, false, p->L, p->P_ws, 64))
     return STARK_EUNSUPPORTED;
+  // planes for the products: the digit products' where the plan has them
+  if (!p->int_m && p->n > 0) {
+    p->int_m = p->limb_m;
+    if (!p->int_m) {
+      const size_t bytes = (size_t)p->P * p->L * p->L * sizeof(float);
+      if (cudaMalloc(&p->int_m, bytes) == cudaSuccess) {
+        p->ws_bytes += (int64_t)bytes;
+      } else {  // without them the products are added into C as they finish
+        cudaGetLastError();
+        p->int_m = nullptr;
+      }
+    }
+    if (p->int_m && !make_tmap_mplanes(&p->tmIM, p->int_m, p->L, p->P)) return STARK_EUNSUPPORTED;
+  }
   p->int_bound = max_abs;
   p->int_tc = true;
   return STARK_OK;
@@ -1051,6 +1065,7 @@ void plan_release(stark_plan_s* p) {
   cudaFree(p->cstage);
   cudaFree(p->m_planes);
   cudaFree(p->q_planes);
+  if (p->int_m != p->limb_m) cudaFree(p->int_m);
   cudaFree(p->limb_m);
   cudaFree(p->limb_aux);
   for (auto e : p->ev)
@@ -1068,8 +1083,10 @@ static stark_status to_status(cudaError_t e) {
 // Divide phase into the workspace.  top < 0: every leaf operand (breadth
 // first); top = i1: only the subtree below top-level product M_{i1+1}
 // (depth-first traversal), its leaves in planes 0..7^(d-1)-1.
-stark_status plan_divide_top(stark_plan_s* p, const void* A, const void* B, cudaStream_t s, int top, int levels,
-                             int64_t plane_off) {
+// With `zero`, zero_bytes there are cleared too (a split plan's C or staging
+// copy, ahead of a combine that adds into it).
+static stark_status plan_divide_top(stark_plan_s* p, const void* A, const void* B, cudaStream_t s, int top, int levels,
+                                    int64_t plane_off, void* zero = nullptr, size_t zero_bytes = 0) {
   if (!p->X || !p->Y) return STARK_ENOMEM;  // no workspace (failed reallocation)
   // depth first: the subtree below `levels` top levels along the M-index path `top`
   const int lv = top >= 0 ? levels : 0;
@@ -1095,7 +1112,14 @@ stark_status plan_divide_top(stark_plan_s* p, const void* A, const void* B, cuda
     db.out_lo = static_cast<char*>(p->Y) + half + off;
   }
   stark_status st = STARK_OK;
-  if (top < 0 && depth == 3 && (om == kOutSplitBf16 || om == kOutSplitTf32 || om == kOutSplitFp16) &&
+  const bool pair = top < 0 && depth <= 2 && p->is_tc;
+  if (zero && (!pair || (reinterpret_cast<uintptr_t>(zero) & 15) != 0)) {
+    if (cudaMemsetAsync(zero, 0, zero_bytes, s) != cudaSuccess) return to_status(cudaGetLastError());
+    zero = nullptr;
+  }
+  if (pair) {
+    st = to_status(launch_divide_pair(da, db, depth, om, zero, (int64_t)zero_bytes, s));
+  } else if (top < 0 && depth == 3 && (om == kOutSplitBf16 || om == kOutSplitTf32 || om == kOutSplitFp16) &&
       divide_staged_fits(p->L)) {
     // breadth first at depth 3, split fp32: one pass per operand, the
     // input tile staged in shared memory
@@ -1140,6 +1164,12 @@ static stark_status plan_divide_shard(stark_plan_s* p, const void* A, const void
   return st;
 }
 
+stark_status plan_divide_clear(stark_plan_s* p, const void* A, const void* B, void* zero, size_t zero_bytes,
+                               cudaStream_t s) {
+  if (p->dfs || p->shard_levels) return STARK_EUNSUPPORTED;
+  return plan_divide_top(p, A, B, s, -1, 0, 0, zero, zero_bytes);
+}
+
 stark_status plan_divide(stark_plan_s* p, const void* A, const void* B, cudaStream_t s) {
   if (p->dfs) return STARK_EUNSUPPORTED;  // the workspace holds one subtree only
   if (p->shard_levels) return plan_divide_shard(p, A, B, s, p->shard_lb, p->shard_le);
@@ -1173,11 +1203,43 @@ static bool plan_limb_stored(const stark_plan_s* p, int64_t lb, int64_t le) {
   return plan_limbs(p) && lb == 0 && le == p->P;
 }
 
+// The same for the bounded integer leaves.
+static bool plan_int_stored(const stark_plan_s* p, int64_t lb, int64_t le) {
+  return p->int_tc && p->int_m && !p->dfs && !p->shard_levels && lb == 0 && le == p->P;
+}
+
 // Whether a separate pass writes every element of C (combine modes 2 and 3,
-// limb leaves):
+// limb leaves, bounded integers):
 // then C is not cleared first and no staging copy is used.
 static bool plan_stored(const stark_plan_s* p, int64_t lb, int64_t le) {
-  return plan_deterministic(p, lb, le) || plan_sib(p, lb, le) || plan_limb_stored(p, lb, le);
+  return plan_deterministic(p, lb, le) || plan_sib(p, lb, le) || plan_limb_stored(p, lb, le) || plan_int_stored(p, lb, le);
+}
+
+// Whether the fused combine goes through TMA: C, or its staging copy, is a
+// target that tensor maps can address.
+static bool plan_tma_c(const stark_plan_s* p, const void* C) {
+  return p->is_tc && p->combine_mode == 0 && (plan_uses_cstage(p, C) || c_is_tma_target(C, p->n));
+}
+
+// Slices of every tile's K range: while the leaves' tiles fill at most half of
+// the units that run at once (CTA pairs, or CTAs), each tile is cut in two
+// again, its slices adding into C like tiles of other leaves.  n = 256 has one
+// tile of 256 x 256; whole it took 12.4 us of leaf kernel.
+static int plan_ksplit(const stark_plan_s* p, const void* C, int64_t lb, int64_t le) {
+  if (!plan_tma_c(p, C) || p->promo_k || p->deep_pipeline || p->dfs || p->shard_levels) return 1;
+  const bool wide = p->pair_mode == 2 && p->bn == 256;
+  const int64_t tm = p->L / (wide ? 256 : 128), tn = p->L / p->bn;
+  const int64_t items = (le - lb) * tm * tn, units = wide ? p->num_sms / 2 : p->num_sms;
+  const int64_t kblocks = p->L / (p->dt == STARK_F32_SPLIT_TF32 ? 32 : 64);
+  int ks = 1;
+  while (kblocks % (2 * ks) == 0 && items * 2 * ks <= units) ks *= 2;
+  return ks;
+}
+
+// Whether every element of C gets exactly one contribution (one leaf, whole K
+// ranges), stored instead of added into a cleared C.
+static bool plan_direct(const stark_plan_s* p, const void* C, int64_t lb, int64_t le) {
+  return p->depth == 0 && lb == 0 && le == 1 && plan_tma_c(p, C) && plan_ksplit(p, C, lb, le) == 1;
 }
 
 // Leaf products of leaves [lb, le) with the combine, operands in workspace
@@ -1207,6 +1269,11 @@ static stark_status plan_leaves(stark_plan_s* p, void* C, int64_t lb, int64_t le
     CUtensorMap tmC;
     std::memset(&tmC, 0, sizeof(tmC));
     a.use_tma_c = (p->combine_mode == 0 && make_tmap_c(&tmC, a.C, core_side(p), a.ldc)) ? 1 : 0;
+    if (a.use_tma_c) {
+      a.ksplit = plan_ksplit(p, C, lb, le);
+      if (plan_direct(p, C, lb, le)) a.use_tma_c = 2;
+    }
+    a.pdl = !p->dfs && !p->shard_levels && p->depth <= 2 ? 1 : 0;  // after launch_divide_pair
     if (deterministic) {
       a.store_m = 1;
       a.use_tma_c = 0;
@@ -1278,7 +1345,18 @@ static stark_status plan_leaves(stark_plan_s* p, void* C, int64_t lb, int64_t le
     a.n = core_side(p);
     a.err = p->d_err;
     a.timeout_ns = p->timeout_ns;
-    st = to_status(launch_leaf_tc_int(a, &p->tmAi, &p->tmBi, p->int_bn, p->num_sms, s));
+    const bool stored = plan_int_stored(p, lb, le);
+    a.store_m = stored ? 1 : 0;
+    CUtensorMap none;
+    std::memset(&none, 0, sizeof(none));
+    st = to_status(launch_leaf_tc_int(a, &p->tmAi, &p->tmBi, stored ? &p->tmIM : &none, p->int_bn, p->num_sms, s));
+    if (st == STARK_OK && stored) {
+      if (cudaEvent_t* ev = plan_timing_events(p)) {
+        cudaEventRecord(ev[3], s);  // the leaf products end, the combine pass starts
+        p->timing_leaf_marked = true;
+      }
+      st = to_status(launch_combine_limb(p->int_m, p->depth, p->L, core_side(p), C, p->n, p->X, kInF32, s));
+    }
   } else {
     LeafCcArgs a{};
     a.P = (int32_t)p->P_ws;
@@ -1347,14 +1425,13 @@ static stark_status plan_limb_leaves(stark_plan_s* p, const void* A, const void*
     p->timing_leaf_marked = true;
   }
   if (st == STARK_OK && stored && p->depth > 0)
-    st = to_status(launch_combine_limb(p->limb_m, p->depth, p->L, core_side(p), C, p->n, p->X, f64, s));
+    st = to_status(launch_combine_limb(p->limb_m, p->depth, p->L, core_side(p), C, p->n, p->X,
+                                       f64 ? kInF64 : kInI64, s));
   if (st != STARK_OK || !f64) return st;
-  st = to_status(launch_gated_clear(C, core_side(p), p->n, p->d_flag, p->num_sms, s));
-  for (int side = 0; side < 2 && st == STARK_OK; ++side) {
-    DivideArgs d{side ? B : A, core_side(p), p->npad, p->L, side ? p->Y : p->X, nullptr, p->d_err, -1, p->n};
-    d.gate = p->d_flag;
-    st = to_status(launch_divide(d, p->depth, side, kInF64, kOutPlain, s));
-  }
+  DivideArgs da{A, core_side(p), p->npad, p->L, p->X, nullptr, p->d_err, -1, p->n};
+  DivideArgs db{B, core_side(p), p->npad, p->L, p->Y, nullptr, p->d_err, -1, p->n};
+  da.gate = db.gate = p->d_flag;
+  st = to_status(launch_redo_divide(da, db, p->depth, C, s));
   if (st != STARK_OK) return st;
   LeafCcArgs c{};
   c.P = (int32_t)p->P;
@@ -1405,8 +1482,9 @@ static stark_status plan_border(stark_plan_s* p, const void* A, const void* B, v
   return STARK_OK;
 }
 
-stark_status plan_run_accumulate(stark_plan_s* p, const void* A, const void* B, void* C, int64_t lb, int64_t le,
-                                 cudaStream_t s) {
+// `zero`: zero_bytes for the divide to clear first (C, or its staging copy).
+static stark_status plan_run_accumulate(stark_plan_s* p, const void* A, const void* B, void* C, int64_t lb, int64_t le,
+                                        cudaStream_t s, void* zero, size_t zero_bytes) {
   if (p->n == 0) return STARK_OK;
   if (!A || !B || !C) return STARK_EINVAL;
   if (!p->X || !p->Y) return STARK_ENOMEM;  // a failed workspace reallocation left none
@@ -1435,7 +1513,7 @@ stark_status plan_run_accumulate(stark_plan_s* p, const void* A, const void* B, 
     if (ev) cudaEventRecord(ev[2], s);
     st = plan_limb_leaves(p, A, B, C, lb, le, s);
   } else if (!p->dfs) {
-    st = plan_divide_top(p, A, B, s, -1, 0, 0);
+    st = plan_divide_top(p, A, B, s, -1, 0, 0, zero, zero_bytes);
     if (st != STARK_OK) return st;
     if (ev) cudaEventRecord(ev[2], s);
     st = plan_leaves(p, C, lb, le, 0, s);
@@ -1484,15 +1562,18 @@ stark_status plan_run(stark_plan_s* p, const void* A, const void* B, void* C, in
     ++p->timing_used;
     p->timing_active = true;
   }
-  if (plan_stored(p, lb, le)) {
-    // a separate combine pass writes every element of C: nothing to clear
-  } else if (p->is_tc && plan_uses_cstage(p, C)) {
-    if (cudaMemsetAsync(p->cstage, 0, (size_t)p->n * staged_ld(p->n) * 4, s) != cudaSuccess)
-      return to_status(cudaGetLastError());
-  } else if (cudaMemsetAsync(C, 0, (size_t)p->n * p->n * p->esz, s) != cudaSuccess) {
-    return to_status(cudaGetLastError());
+  if (plan_stored(p, lb, le) || (plan_direct(p, C, lb, le) && !p->dfs && !p->shard_levels)) {
+    // a separate combine pass, or the leaf kernel itself, writes every
+    // element of C: nothing to clear
+    return plan_run_accumulate(p, A, B, C, lb, le, s, nullptr, 0);
   }
-  return plan_run_accumulate(p, A, B, C, lb, le, s);
+  const bool staged = p->is_tc && plan_uses_cstage(p, C);
+  void* target = staged ? p->cstage : C;
+  const size_t bytes = staged ? (size_t)p->n * staged_ld(p->n) * 4 : (size_t)p->n * p->n * p->esz;
+  if (p->is_tc && !p->dfs && !p->shard_levels && lb < le)  // the divide clears it
+    return plan_run_accumulate(p, A, B, C, lb, le, s, target, bytes);
+  if (cudaMemsetAsync(target, 0, bytes, s) != cudaSuccess) return to_status(cudaGetLastError());
+  return plan_run_accumulate(p, A, B, C, lb, le, s, nullptr, 0);
 }
 
 stark_status plan_ensure_cstage(stark_plan_s* p) {
@@ -1512,9 +1593,8 @@ bool plan_uses_cstage(const stark_plan_s* p, const void* C) {
 }
 
 stark_status plan_copy_cstage(const stark_plan_s* p, void* C, cudaStream_t s) {
-  const size_t w = (size_t)p->n * 4;
-  return to_status(cudaMemcpy2DAsync(C, w, p->cstage, (size_t)staged_ld(p->n) * 4, w, (size_t)p->n,
-                                     cudaMemcpyDeviceToDevice, s));
+  return to_status(launch_unstage(static_cast<const float*>(p->cstage), staged_ld(p->n), static_cast<float*>(C), p->n,
+                                  p->num_sms, s));
 }
 
 }  // namespace stark

@@ -76,6 +76,8 @@ struct stark_plan_s {
   int64_t int_bound = 0;
   bool int_tc = false;
   int int_bn = 128;
+  void* int_m = nullptr;  // [P][L][L] fp32 products of a whole breadth-first product (null: added into C)
+  CUtensorMap tmIM;
   CUtensorMap tmAi, tmBi;
   // I64 and F64 leaves as digit products on the tensor cores (leaf_limb.cu):
   // breadth first, leaf sides >= 128; X and Y then hold 16 bytes per element
@@ -156,7 +158,8 @@ bool plan_uses_cstage(const stark_plan_s* p, const void* C);
 stark_status plan_copy_cstage(const stark_plan_s* p, void* C, cudaStream_t s);
 // Divide phase only: all leaf operands of A and B into the workspace.
 stark_status plan_divide(stark_plan_s* p, const void* A, const void* B, cudaStream_t s);
-// The same without zeroing C first (C accumulates).
-stark_status plan_run_accumulate(stark_plan_s* p, const void* A, const void* B, void* C, int64_t lb, int64_t le,
-                                 cudaStream_t s);
+// The same for a breadth-first split plan, with zero_bytes at `zero` (may be
+// null) cleared ahead of a combine that adds there.
+stark_status plan_divide_clear(stark_plan_s* p, const void* A, const void* B, void* zero, size_t zero_bytes,
+                               cudaStream_t s);
 }  // namespace stark

@@ -55,6 +55,7 @@ struct Request {
   stark_plan_s* ws = nullptr;  // workspace while running
   void* target = nullptr;      // combine target: C, or the workspace's staging copy
   int64_t ld = 0;              // its row pitch
+  bool direct = false;         // its elements are stored once (one leaf), not added
   stark_status status = STARK_OK;
   bool deferred = false;       // admission waited at least once for device memory
 };
@@ -268,8 +269,9 @@ stark_status launch_micro_batch(stark_server_s* s, Slot& slot, std::vector<Reque
     if (split && !r->ws->dfs) {
       r->target = staged ? r->ws->cstage : r->C;
       r->ld = staged ? staged_ld(r->n) : r->n;
-      if (cudaMemsetAsync(r->target, 0, (size_t)r->n * r->ld * sizeof(float), st) != cudaSuccess) return STARK_ECUDA;
-      e = plan_divide(&view, r->A, r->B, st);
+      CUtensorMap probe;  // (one leaf and a C that TMA addresses: stored, not added into a cleared C)
+      r->direct = r->ws->depth == 0 && make_tmap_c(&probe, r->target, r->n, r->ld);
+      e = plan_divide_clear(&view, r->A, r->B, r->direct ? nullptr : r->target, (size_t)r->n * r->ld * sizeof(float), st);
       tc.push_back(r);
     } else {
       // plain dtypes, and depth-first workspaces (one subtree's operands at a
@@ -310,7 +312,7 @@ stark_status launch_micro_batch(stark_server_s* s, Slot& slot, std::vector<Reque
       g.C = static_cast<float*>(tc[k]->target);
       g.n = tc[k]->n;
       g.ldc = tc[k]->ld;
-      g.use_tma_c = make_tmap_c(&g.tmC, g.C, g.n, g.ldc) ? 1 : 0;
+      g.use_tma_c = make_tmap_c(&g.tmC, g.C, g.n, g.ldc) ? (tc[k]->direct ? 2 : 1) : 0;
       items += bn == 256 ? p->P * (p->L / 256) * (p->L / 256) : p->P * (p->L / 128) * (p->L / 128);
     }
     if (split == (int)tc.size()) {
@@ -339,9 +341,8 @@ stark_status launch_micro_batch(stark_server_s* s, Slot& slot, std::vector<Reque
     }
     for (Request* r : tc)
       if (r->target != r->C) {
-        const size_t w = (size_t)r->n * sizeof(float);
-        if (cudaMemcpy2DAsync(r->C, w, r->target, (size_t)r->ld * sizeof(float), w, (size_t)r->n,
-                              cudaMemcpyDeviceToDevice, st) != cudaSuccess)
+        if (launch_unstage(static_cast<const float*>(r->target), r->ld, static_cast<float*>(r->C), r->n, s->num_sms,
+                           st) != cudaSuccess)
           return STARK_ECUDA;
       }
   }

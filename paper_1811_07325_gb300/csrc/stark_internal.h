@@ -79,7 +79,7 @@ struct DivideArgs {
                       // full padded side >> top_levels)
   int64_t ld;         // row stride of X in elements (>= n)
   int top_levels;     // levels above the subtree (1, or 2 for the split dtypes) when top >= 0
-  const int* gate;    // not null: the launch does nothing unless *gate != 0
+  const int* gate;    // launch_redo_divide only: does nothing unless *gate != 0
   // kOutLimbs, F64 input: exponents [leaf][L] of the operand's rows (side 0)
   // or columns (side 1), and the digit-magnitude planes of the first 128 of K
   // ([leaf][L][128] for side 0, [leaf][128][L] for side 1)
@@ -90,6 +90,10 @@ struct DivideArgs {
 // Divide phase for one operand: writes the 7^depth leaf operand sums as
 // row-major L x L planes.  side 0 = A (M x K planes), side 1 = B (K x N).
 cudaError_t launch_divide(const DivideArgs& a, int depth, int side, InType in, OutMode out, cudaStream_t s);
+// Both operands of a split dtype, breadth first at depth <= 2, in one launch
+// that can also clear zero_bytes (a multiple of 4) at the 16-byte aligned `zero`.
+cudaError_t launch_divide_pair(const DivideArgs& a, const DivideArgs& b, int depth, OutMode out, void* zero,
+                               int64_t zero_bytes, cudaStream_t s);
 // The same for a depth-first subtree (a.top >= 0); launch_divide forwards.
 cudaError_t launch_divide_top(const DivideArgs& a, int depth, int side, InType in, OutMode out, cudaStream_t s);
 // Depth 3, split-fp32 outputs, breadth first (a.top < 0): one pass per
@@ -116,8 +120,9 @@ struct LimbBoundsArgs {
   int* flag;          // cleared, then set for infinities, NaN and exponents outside +-400
 };
 cudaError_t launch_limb_bounds(const LimbBoundsArgs& a, cudaStream_t s);
-// C = 0 where *gate != 0 (n x n elements of 8 bytes, row stride ld).
-cudaError_t launch_gated_clear(void* C, int64_t n, int64_t ld, const int* gate, int num_sms, cudaStream_t s);
+// Where *a.gate != 0: the plain fp64 operands of both sides (X planes, breadth
+// first) and a cleared C (a.n x a.n, row stride a.ld); else nothing.
+cudaError_t launch_redo_divide(const DivideArgs& a, const DivideArgs& b, int depth, void* C, cudaStream_t s);
 
 // C (+)= A B on sub-blocks (M x K times K x N, row strides lda, ldb, ldc in
 // elements) on the CUDA cores: the edges of a peeled product.  Element type
@@ -146,6 +151,8 @@ bool make_tmap_mplanes(CUtensorMap* m, void* base, int64_t L, int64_t planes);
 // [planes][rows][cols] of 16-bit elements; boxes of 64 or 32 columns (128- or 64-byte swizzle).
 bool make_tmap_half3(CUtensorMap* m, void* base, int64_t cols, int64_t rows, int64_t planes, int box_cols, int box_rows,
                      int box_planes);
+// C (row pitch n) = the n x n staging copy `src` of row pitch ld.
+cudaError_t launch_unstage(const float* src, int64_t ld, float* C, int64_t n, int num_sms, cudaStream_t s);
 // In-place transpose of `count` square L x L fp32 planes.
 cudaError_t launch_transpose_planes(float* planes, int64_t L, int64_t count, cudaStream_t s);
 
@@ -178,7 +185,10 @@ struct LeafTcArgs {
   int64_t n;
   int* err;
   uint64_t timeout_ns;
-  int32_t use_tma_c;   // 1: combine by TMA bulk add-reductions through tmC
+  int32_t use_tma_c;   // 1: combine by TMA bulk add-reductions through tmC; 2: one leaf, plain TMA stores
+  int32_t ksplit;      // > 1 (one problem, use_tma_c 1): every tile's K range in this many equal
+                       // slices, each an item of its own that adds into C
+  int32_t pdl;         // 1: programmatic dependent launch (the stream's previous kernel is a divide)
   int32_t pair;        // 2: cta_group::2 pair MMA where the tiling allows; 0: single CTAs
   int32_t row_bytes;   // swizzled smem row of the operand tiles: 128 or 64 (tensor maps must match)
   int32_t store_m;     // 1: store each leaf tile to the M planes (tmC = their map) instead of combining
@@ -209,8 +219,9 @@ cudaError_t launch_leaf_tc(const LeafTcArgs& a, const CUtensorMap* tmA, const CU
                            const CUtensorMap* tmC, bool tf32, int bn, int num_sms, cudaStream_t s);
 // Exact integer leaves: one bf16 product per K step over [P][L][L] bf16
 // planes holding integers, combined into an int64 C (a.C reinterpreted).
-cudaError_t launch_leaf_tc_int(const LeafTcArgs& a, const CUtensorMap* tmA, const CUtensorMap* tmB, int bn,
-                               int num_sms, cudaStream_t s);
+// With a.store_m the products go to the fp32 planes that tmC maps instead.
+cudaError_t launch_leaf_tc_int(const LeafTcArgs& a, const CUtensorMap* tmA, const CUtensorMap* tmB,
+                               const CUtensorMap* tmC, int bn, int num_sms, cudaStream_t s);
 // Grouped single-CTA launch over a.groups (tensor maps taken from the
 // descriptors), 128 x 128 tiles (bn == 128 only).
 cudaError_t launch_leaf_tc_grouped(const LeafTcArgs& a, bool tf32, int bn, int num_sms, cudaStream_t s);
@@ -268,10 +279,12 @@ cudaError_t launch_leaf_limb(const LeafLimbArgs& a, const CUtensorMap* tmA, cons
                              const CUtensorMap* tmSA, const CUtensorMap* tmSB, bool f64, int num_sms,
                              cudaStream_t s);
 
-// Ordered combine of the stored limb products M [7^depth][L][L] into C (depth
-// 1..4); tmp: 7^(depth - 2) (4 L)^2 elements for depths 3 and 4.
+// Ordered combine of stored leaf products M [7^depth][L][L] into a C of 8-byte
+// elements (depth 0..4): fp64 (kInF64), int64 (kInI64), or integers held in
+// fp32 into int64 (kInF32).  tmp: 7^(depth - 2) (4 L)^2 elements of C's type
+// for depths 3 and 4.
 cudaError_t launch_combine_limb(const void* M, int depth, int64_t L, int64_t n, void* C, int64_t ldc, void* tmp,
-                                bool f64, cudaStream_t s);
+                                InType t, cudaStream_t s);
 
 cudaError_t launch_wait_selftest(int* err, uint64_t timeout_ns, cudaStream_t s);
 

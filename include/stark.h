@@ -375,16 +375,17 @@ typedef struct stark_batch_s *stark_batch_t;
 /* A batch of `count` independent products C_i = A_i * B_i of sizes n[i] (any
  * mix), one tensor-core dtype (F32_SPLIT_BF16, F32_SPLIT_TF32 or
  * F32_SPLIT_FP16).  Every leaf
- * product of every member (Alg. 4) is a work item of ONE persistent grouped
+ * product of every member (Alg. 4) is a work item of a persistent grouped
  * leaf launch, whose epilogue combines (Alg. 5) into each member's own C;
- * the member divides (Alg. 3) precede it.  The launch sequence is recorded
+ * its members' divides (Alg. 3) precede it.  The launch sequence is recorded
  * in a CUDA graph on first use and replayed while the pointers stay the
  * same.  depth = -1: each member's depth and leaf tile are chosen by the
  * autotuner, which times the candidate (depth, tile) pairs on the device
  * (cached per size class and dtype for the process); otherwise members
  * whose leaf side allows it use 256-wide tiles.  Members on 256-wide tiles
- * share one grouped launch of CTA pairs, the others a second one with
- * 128-wide tiles on single CTAs.  Allocates every member's workspace.
+ * share up to three grouped launches of CTA pairs (the later ones' divides run
+ * under the earlier ones' products), the others one with 128-wide tiles on
+ * single CTAs.  Allocates every member's workspace.
  * Errors: EINVAL (count <= 0 or > 4096, n[i] <= 0, depth out of range),
  * EUNSUPPORTED (other dtypes, not a GB300), ENOMEM, ECUDA. */
 STARK_API stark_status stark_batch_create(int32_t count, const int64_t *n, int depth, stark_dtype dtype,

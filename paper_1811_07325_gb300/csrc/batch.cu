@@ -1,21 +1,20 @@
 // batch.cu -- many independent products in one grouped, graph-captured pass.
 //
 // Each member keeps its own plan (operand planes, C-target table, operand
-// tensor maps).  One stark_batch_mul enqueues, for every member, the zeroing
-// of C and the divide of A and B, then ONE persistent grouped leaf launch
-// whose work items are all (member, leaf, tile) triples: the 7^d leaf
-// products of every member share the GPU in a single launch, and each
-// item's epilogue combines into its own member's C.  The whole sequence is
-// captured once in a CUDA graph and replayed while the pointers are
-// unchanged.
+// tensor maps).  One stark_batch_mul enqueues, for every member, the divide of
+// A and B with the clearing of C, and a few persistent grouped leaf launches
+// whose work items are (member, leaf, tile) triples: the 7^d leaf products of
+// their members share the GPU, and each item's epilogue combines into its own
+// member's C.  The whole sequence is captured once in a CUDA graph and
+// replayed while the pointers are unchanged.
 //
 // Depth per member: given, or chosen by the autotuner, which times the
 // candidate (depth, leaf tile) pairs on the device (one warm-up and three
 // timed products per candidate on scratch inputs) and caches the winner per
 // size class and dtype for the process.  The tile candidates are CTA pairs
 // on 256 x 256 tiles (cta_group::2; leaf sides that are multiples of 256)
-// and single CTAs on 128 x 128 tiles.  Members whose tile is 256 share one
-// grouped launch of CTA pairs, the others a second one of single CTAs.
+// and single CTAs on 128 x 128 tiles.  Members whose tile is 256 share up to
+// three grouped launches of CTA pairs, the others one of single CTAs.
 #include <algorithm>
 #include <cstring>
 #include <map>
@@ -129,19 +128,26 @@ int autotune_depth(int64_t n, stark_dtype dt) {
 struct stark_batch_s {
   stark_dtype dt = STARK_F32_SPLIT_BF16;
   int bn = 128;     // 256 when any member runs 256-wide tiles
-  int split = 0;    // members [0, split) run 256-wide tiles, the rest 128-wide
-  int items_wide = 0;
+  // the grouped leaf launches: members [first, first + count) of the sorted
+  // order, whose items are numbered from 0; the 256-wide ones come first
+  struct Launch {
+    int first, count, items;
+    bool wide;
+  };
+  std::vector<Launch> launches;
   std::vector<stark_plan_s*> plans;
   std::vector<stark::GroupDesc> host_desc;
   stark::GroupDesc* d_desc = nullptr;
-  int total_items = 0;
+  int64_t total_items = 0;
   int* d_err = nullptr;
   cudaStream_t cap = nullptr;  // private capture stream
   // the members' clears and divides are captured on kForks side streams
   // forked from `cap`, so the graph runs them concurrently (small members'
   // kernels are launch- and latency-bound one after another)
   static constexpr int kForks = 8;
+  static constexpr int kMaxLaunches = 4;
   cudaStream_t side[kForks] = {};
+  cudaStream_t leaf[kMaxLaunches] = {};  // branches of the leaf launches
   cudaEvent_t fork_ev = nullptr;
   cudaEvent_t join_ev[kForks] = {};
   cudaGraphExec_t exec = nullptr;
@@ -166,6 +172,8 @@ static void batch_free(stark_batch_s* b) {
     if (b->side[i]) cudaStreamDestroy(b->side[i]);
     if (b->join_ev[i]) cudaEventDestroy(b->join_ev[i]);
   }
+  for (cudaStream_t l : b->leaf)
+    if (l) cudaStreamDestroy(l);
   if (b->fork_ev) cudaEventDestroy(b->fork_ev);
   cudaGetLastError();
   delete b;
@@ -206,53 +214,72 @@ stark_status stark_batch_create(int32_t count, const int64_t* n, int depth, star
     batch_free(b);
     return st;
   }
-  // two grouped launches: members on 256-wide tiles (CTA pairs) first, then
-  // the rest on 128-wide tiles; largest products first in each
+  // members on 256-wide tiles (CTA pairs) first, then the rest on 128-wide
+  // tiles; largest products first in each
   const std::vector<int> tiles = b->tiles;
   auto wide = [&](int i) { return tiles[i] == 256; };
   std::sort(order.begin(), order.end(), [&](int x, int y) {
     if (wide(x) != wide(y)) return wide(x);
     return b->plans[x]->n > b->plans[y]->n;
   });
-  b->split = 0;
-  while (b->split < count && wide(order[b->split])) ++b->split;
-  b->bn = b->split > 0 ? 256 : 128;
+  int split = 0;
+  while (split < count && wide(order[split])) ++split;
+  b->bn = split > 0 ? 256 : 128;
+  // The 256-wide members in up to three launches, so that the divides of the
+  // later ones run under the leaf products of the earlier ones (a leaf kernel
+  // leaves the SMs threads and registers for them).  The first gets an eighth
+  // of the work, the second three eighths: its divides take a quarter to a
+  // third of its leaf time.  Not when all the divides together move less than
+  // 256 MB, about 40 us.
+  int64_t divide_bytes = 0;
+  double work = 0;
+  auto leaf_work = [&](const stark_plan_s* p) { return (double)p->P * p->L * p->L * p->L; };
+  for (int k = 0; k < split; ++k) {
+    const stark_plan_s* p = b->plans[order[k]];
+    divide_bytes += 2 * p->n * p->n * 4 + operand_bytes(p->n, p->depth, dt);
+    work += leaf_work(p);
+  }
+  std::vector<int> cuts;  // ends of the launches
+  if (divide_bytes >= (int64_t)256 << 20) {
+    double done = 0;
+    for (int k = 0; k + 1 < split && cuts.size() < 2; ++k) {
+      done += leaf_work(b->plans[order[k]]);
+      if (done >= work * (cuts.empty() ? 0.125 : 0.5)) cuts.push_back(k + 1);
+    }
+  }
+  if (split > 0) cuts.push_back(split);
+  if (split < count) cuts.push_back(count);
   b->host_desc.resize(count);
-  int64_t items = 0, items_wide = 0;
-  for (int k = 0; k < count; ++k) {
-    if (k == b->split) {
-      items_wide = items;
-      items = 0;  // the second launch numbers its own items
+  int first = 0;
+  for (int end : cuts) {
+    int64_t items = 0;
+    for (int k = first; k < end; ++k) {
+      stark_plan_s* p = b->plans[order[k]];
+      const int bn = k < split ? 256 : 128;
+      GroupDesc& g = b->host_desc[k];
+      std::memset(&g, 0, sizeof(g));
+      g.tmA = p->tmA;
+      if (dt == STARK_F32_SPLIT_TF32 && !p->tf32_mn) {
+        // K-major tf32 Y; 256-wide members run CTA pairs: each CTA loads 128 Y rows
+        if (!make_tmap_planes(&g.tmB, p->Y, true, p->L, 2 * p->P, bn == 256 ? 128 : bn)) st = STARK_EUNSUPPORTED;
+      } else {
+        g.tmB = p->tmB;
+      }
+      g.item_base = (int32_t)items;
+      g.P = (int32_t)p->P;
+      g.L = (int32_t)p->L;
+      g.ctab = p->d_ctab;
+      g.ccount = p->d_ccount;
+      g.maxT = p->maxT;
+      g.n = p->n;
+      // 256-wide members: 256 x 256 pair tiles (CTA pairs); others 128 x 128
+      items += bn == 256 ? p->P * (p->L / 256) * (p->L / 256) : p->P * (p->L / 128) * (p->L / 128);
     }
-    stark_plan_s* p = b->plans[order[k]];
-    const int bn = k < b->split ? 256 : 128;
-    GroupDesc& g = b->host_desc[k];
-    std::memset(&g, 0, sizeof(g));
-    g.tmA = p->tmA;
-    if (dt == STARK_F32_SPLIT_TF32 && !p->tf32_mn) {
-      // K-major tf32 Y; 256-wide members run CTA pairs: each CTA loads 128 Y rows
-      if (!make_tmap_planes(&g.tmB, p->Y, true, p->L, 2 * p->P, bn == 256 ? 128 : bn)) st = STARK_EUNSUPPORTED;
-    } else {
-      g.tmB = p->tmB;
-    }
-    g.item_base = (int32_t)items;
-    g.P = (int32_t)p->P;
-    g.L = (int32_t)p->L;
-    g.ctab = p->d_ctab;
-    g.ccount = p->d_ccount;
-    g.maxT = p->maxT;
-    g.n = p->n;
-    // 256-wide members: 256 x 256 pair tiles (CTA pairs); others 128 x 128
-    items += bn == 256 ? p->P * (p->L / 256) * (p->L / 256) : p->P * (p->L / 128) * (p->L / 128);
+    if (items > 0x7FFFFFFF) st = STARK_EINVAL;
+    b->launches.push_back({first, end - first, (int)items, first < split});
+    b->total_items += items;
+    first = end;
   }
-  if (b->split == count) {
-    items_wide = items;
-    items = 0;
-  }
-  if (items_wide > 0x7FFFFFFF) st = STARK_EINVAL;
-  b->items_wide = (int)items_wide;
-  if (items > 0x7FFFFFFF) st = STARK_EINVAL;
-  b->total_items = (int)items;  // items of the 128-wide launch
   // keep the member order used by the descriptors
   std::vector<stark_plan_s*> sorted(count);
   for (int k = 0; k < count; ++k) sorted[k] = b->plans[order[k]];
@@ -267,6 +294,8 @@ stark_status stark_batch_create(int32_t count, const int64_t* n, int depth, star
     if (cudaStreamCreateWithFlags(&b->side[i], cudaStreamNonBlocking) != cudaSuccess ||
         cudaEventCreateWithFlags(&b->join_ev[i], cudaEventDisableTiming) != cudaSuccess)
       st = STARK_ENOMEM;
+  for (size_t i = 0; i < b->launches.size() && st == STARK_OK; ++i)
+    if (cudaStreamCreateWithFlags(&b->leaf[i], cudaStreamNonBlocking) != cudaSuccess) st = STARK_ENOMEM;
   if (st != STARK_OK) {
     batch_free(b);
     return st;
@@ -305,7 +334,7 @@ stark_status stark_batch_info(stark_batch_t b, int32_t* tile_n, int64_t* work_it
                               int64_t* graph_replays) {
   if (!b) return STARK_EINVAL;
   if (tile_n) *tile_n = b->bn;
-  if (work_items) *work_items = (int64_t)b->total_items + b->items_wide;
+  if (work_items) *work_items = b->total_items;
   if (workspace_bytes) {
     int64_t w = 0;
     for (auto* p : b->plans) w += p->ws_bytes;
@@ -351,55 +380,53 @@ stark_status stark_batch_mul(stark_batch_t b, const void* const* A, const void* 
     cudaGraph_t graph = nullptr;
     if (cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return STARK_ECUDA;
     stark_status st = STARK_OK;
-    // fork: members' clears and divides on the side streams, joined before
-    // the grouped leaf launches
+    // fork: members' clears and divides on the side streams in the order of
+    // the leaf launches, each of which joins its own members' and runs on a
+    // branch of its own (a later launch takes SMs as the tail of an earlier one
+    // frees them)
     constexpr int F = stark_batch_s::kForks;
     if (cudaEventRecord(b->fork_ev, b->cap) != cudaSuccess) st = STARK_ECUDA;
     for (int i = 0; i < F && st == STARK_OK; ++i)
       if (cudaStreamWaitEvent(b->side[i], b->fork_ev, 0) != cudaSuccess) st = STARK_ECUDA;
-    for (int k = 0; k < count && st == STARK_OK; ++k) {
-      stark_plan_s* p = b->plans[k];
-      const GroupDesc& g = b->host_desc[k];
-      cudaStream_t sk = b->side[k % F];
-      st = plan_divide_clear(p, ptrs[3 * k], ptrs[3 * k + 1], g.use_tma_c == 2 ? nullptr : g.C,
-                             (size_t)p->n * g.ldc * sizeof(float), sk);
-    }
-    for (int i = 0; i < F; ++i)  // join (also after an error, so the capture can end)
-      if (cudaEventRecord(b->join_ev[i], b->side[i]) != cudaSuccess ||
-          cudaStreamWaitEvent(b->cap, b->join_ev[i], 0) != cudaSuccess)
-        st = STARK_ECUDA;
-    if (st == STARK_OK) {
+    size_t branches = 0;  // leaf streams that are part of the capture
+    for (size_t q = 0; q < b->launches.size() && st == STARK_OK; ++q) {
+      const auto& run = b->launches[q];
+      for (int k = run.first; k < run.first + run.count && st == STARK_OK; ++k) {
+        stark_plan_s* p = b->plans[k];
+        const GroupDesc& g = b->host_desc[k];
+        st = plan_divide_clear(p, ptrs[3 * k], ptrs[3 * k + 1], g.use_tma_c == 2 ? nullptr : g.C,
+                               (size_t)p->n * g.ldc * sizeof(float), b->side[k % F]);
+      }
+      for (int i = 0; i < F && st == STARK_OK; ++i)
+        if (cudaEventRecord(b->join_ev[i], b->side[i]) != cudaSuccess ||
+            cudaStreamWaitEvent(b->leaf[q], b->join_ev[i], 0) != cudaSuccess)
+          st = STARK_ECUDA;
+        else
+          branches = q + 1;
+      if (st != STARK_OK) break;
       LeafTcArgs a{};
       a.err = b->d_err;
       a.timeout_ns = kDefaultTimeoutNs;
       const bool tf32 = b->dt == STARK_F32_SPLIT_TF32;
       a.b_mn = tf32 && b->plans[0]->tf32_mn;  // every member has the plan default
       a.fp16 = b->dt == STARK_F32_SPLIT_FP16 ? 1 : 0;
-      // the two grouped launches on two branches of the graph: the second
-      // takes SMs as the first one's tail frees them
-      const bool both = b->split > 0 && b->split < count;
-      cudaStream_t s_wide = both ? b->side[0] : b->cap, s_narrow = both ? b->side[1] : b->cap;
-      if (both && (cudaEventRecord(b->fork_ev, b->cap) != cudaSuccess ||
-                   cudaStreamWaitEvent(s_wide, b->fork_ev, 0) != cudaSuccess ||
-                   cudaStreamWaitEvent(s_narrow, b->fork_ev, 0) != cudaSuccess))
+      a.groups = b->d_desc + run.first;
+      a.ngroups = run.count;
+      a.total_items = run.items;
+      if ((run.wide ? launch_leaf_tc2_grouped(a, tf32, device_sm_count(), b->leaf[q])
+                    : launch_leaf_tc_grouped(a, tf32, 128, device_sm_count(), b->leaf[q])) != cudaSuccess)
         st = STARK_ECUDA;
-      if (st == STARK_OK && b->split > 0) {  // 256-wide members
-        a.groups = b->d_desc;
-        a.ngroups = b->split;
-        a.total_items = b->items_wide;
-        if (launch_leaf_tc2_grouped(a, tf32, device_sm_count(), s_wide) != cudaSuccess) st = STARK_ECUDA;
-      }
-      if (st == STARK_OK && b->split < count) {  // 128-wide members
-        a.groups = b->d_desc + b->split;
-        a.ngroups = count - b->split;
-        a.total_items = b->total_items;
-        if (launch_leaf_tc_grouped(a, tf32, 128, device_sm_count(), s_narrow) != cudaSuccess) st = STARK_ECUDA;
-      }
-      if (both)
-        for (int i = 0; i < 2; ++i)
-          if (cudaEventRecord(b->join_ev[i], b->side[i]) != cudaSuccess ||
-              cudaStreamWaitEvent(b->cap, b->join_ev[i], 0) != cudaSuccess)
-            st = STARK_ECUDA;
+    }
+    // join (also after an error, so the capture can end)
+    for (int i = 0; i < F; ++i)
+      if (cudaEventRecord(b->join_ev[i], b->side[i]) != cudaSuccess ||
+          cudaStreamWaitEvent(b->cap, b->join_ev[i], 0) != cudaSuccess)
+        st = STARK_ECUDA;
+    for (size_t q = 0; q < branches; ++q)
+      if (cudaEventRecord(b->fork_ev, b->leaf[q]) != cudaSuccess ||
+          cudaStreamWaitEvent(b->cap, b->fork_ev, 0) != cudaSuccess)
+        st = STARK_ECUDA;
+    if (st == STARK_OK) {
       // members combined into a staging copy: move the result into C
       for (int k = 0; k < count && st == STARK_OK; ++k)
         if (b->host_desc[k].C != ptrs[3 * k + 2])

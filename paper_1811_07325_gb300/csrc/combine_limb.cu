@@ -17,22 +17,30 @@
 // leaf_tc.cu) take the same pass with their own input type: as 64-bit
 // reductions of 256 bytes a row piece from the epilogue, one per target, they
 // kept the copy engine busy for 230 of the 350 us at n = 4096, depth 1.
+#include <type_traits>
+
 #include "stark_internal.h"
 
 namespace stark {
 namespace {
 
-template <typename T>
-struct Pair {
-  T x, y;
+template <typename T, int W>
+struct Cols {
+  T v[W];
 };
-template <typename T>
-__device__ __forceinline__ Pair<T> operator+(const Pair<T>& a, const Pair<T>& b) {
-  return {a.x + b.x, a.y + b.y};
+template <typename T, int W>
+__device__ __forceinline__ Cols<T, W> operator+(const Cols<T, W>& a, const Cols<T, W>& b) {
+  Cols<T, W> r;
+#pragma unroll
+  for (int e = 0; e < W; ++e) r.v[e] = a.v[e] + b.v[e];
+  return r;
 }
-template <typename T>
-__device__ __forceinline__ Pair<T> operator-(const Pair<T>& a, const Pair<T>& b) {
-  return {a.x - b.x, a.y - b.y};
+template <typename T, int W>
+__device__ __forceinline__ Cols<T, W> operator-(const Cols<T, W>& a, const Cols<T, W>& b) {
+  Cols<T, W> r;
+#pragma unroll
+  for (int e = 0; e < W; ++e) r.v[e] = a.v[e] - b.v[e];
+  return r;
 }
 
 // Quadrants of a product from its seven sub-products.
@@ -44,36 +52,43 @@ __device__ __forceinline__ void fold(const V (&m)[7], V (&c)[4]) {
   c[3] = ((m[0] - m[1]) + m[2]) + m[5];
 }
 
-// A thread owns two columns of one position (r, c) of the L x L leaf grid of
-// one product (blockIdx.y) D levels up: 7^D vectors in, 4^D out.
-template <typename T, typename TM, int D>
-__global__ void __launch_bounds__(256, 2)
+// A thread owns W columns of one position (r, c) of the L x L leaf grid of one
+// product (blockIdx.y) D levels up: 7^D vectors in, 4^D out.
+template <typename T, typename TM, int D, int W>
+__global__ void __launch_bounds__(256, W == 1 ? 4 : 2)
     combine_limb_kernel(const TM* __restrict__ M, int64_t L, T* __restrict__ out, int64_t out_plane, int64_t ld, int64_t n) {
-  using V = Pair<T>;
+  using V = Cols<T, W>;
   const int64_t pos = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  if (pos >= L * (L / 2)) return;
-  const int64_t r = pos / (L / 2), c = pos % (L / 2) * 2;
+  if (pos >= L * (L / W)) return;
+  const int64_t r = pos / (L / W), c = pos % (L / W) * W;
   constexpr int P = D == 0 ? 1 : D == 1 ? 7 : 49;
   const TM* src = M + (int64_t)blockIdx.y * P * L * L + r * L + c;
   out += (int64_t)blockIdx.y * out_plane;
   auto load = [&](int leaf) {
+    V x;
     if constexpr (sizeof(TM) == 4) {  // integers held in fp32
-      const float2 x = __ldcs(reinterpret_cast<const float2*>(src + (int64_t)leaf * L * L));
-      return V{(T)(long long)__float2int_rn(x.x), (T)(long long)__float2int_rn(x.y)};
-    } else {
+      static_assert(W == 2, "8-byte loads");
+      const float2 f = __ldcs(reinterpret_cast<const float2*>(src + (int64_t)leaf * L * L));
+      x.v[0] = (T)(long long)__float2int_rn(f.x);
+      x.v[1] = (T)(long long)__float2int_rn(f.y);
+    } else if constexpr (W == 2) {
       const int4 raw = __ldcs(reinterpret_cast<const int4*>(src + (int64_t)leaf * L * L));
-      return *reinterpret_cast<const V*>(&raw);
+      x = *reinterpret_cast<const V*>(&raw);
+    } else {
+      x.v[0] = __ldcs(src + (int64_t)leaf * L * L);
     }
+    return x;
   };
-  const bool vec = (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+  const bool vec = W == 2 && (ld & 1) == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
   auto store = [&](int64_t row, int64_t col, const V& v) {
     if (row >= n || col >= n) return;
     T* dst = out + row * ld + col;
-    if (vec && col + 1 < n) {
+    if (vec && col + W <= n) {
       *reinterpret_cast<int4*>(dst) = *reinterpret_cast<const int4*>(&v);
     } else {
-      dst[0] = v.x;
-      if (col + 1 < n) dst[1] = v.y;
+#pragma unroll
+      for (int e = 0; e < W; ++e)
+        if (col + e < n) dst[e] = v.v[e];
     }
   };
   if constexpr (D == 0) {
@@ -117,9 +132,10 @@ __global__ void __launch_bounds__(256, 2)
 template <typename T, int D, typename TM>
 cudaError_t fold_levels(const TM* M, int64_t L, int64_t products, T* out, int64_t out_plane, int64_t ld, int64_t n,
                         cudaStream_t st) {
-  const int64_t blocks = (L * (L / 2) + 255) / 256;
+  constexpr int W = std::is_same_v<TM, double> && D == 2 ? 1 : 2;
+  const int64_t blocks = (L * (L / W) + 255) / 256;
   if (L % 2 != 0 || blocks > 0x7FFFFFFF || products > 65535) return cudaErrorInvalidValue;
-  combine_limb_kernel<T, TM, D><<<dim3((unsigned)blocks, (unsigned)products), 256, 0, st>>>(M, L, out, out_plane, ld, n);
+  combine_limb_kernel<T, TM, D, W><<<dim3((unsigned)blocks, (unsigned)products), 256, 0, st>>>(M, L, out, out_plane, ld, n);
   count_launch();
   return cudaGetLastError();
 }

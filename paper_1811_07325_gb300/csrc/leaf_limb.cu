@@ -475,15 +475,19 @@ __global__ void __launch_bounds__(kThreadsL, 1)
       const int nt = p.ccount[leaf];
       const CTarget* tg = p.ctab + (int64_t)leaf * p.maxT;
       unsigned long long* C = static_cast<unsigned long long*>(p.C);
-#pragma unroll
+      // (one copy of this code, the next 8 columns' sums moving down: unrolled
+      // over the 64 columns it was 40 KB that every tile fetched anew)
+#pragma unroll 1
       for (int j = 0; j < 8; ++j) {
         unsigned long long v[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           // (a zero row or column has a zero sum, whatever its exponent says)
-          v[e] = F64 ? scaled_double_bits(sum[j * 8 + e], ea + fexp(j * 8 + e) + p.shift - 68)
-                     : (unsigned long long)sum[j * 8 + e];
+          v[e] = F64 ? scaled_double_bits(sum[e], ea + fexp(j * 8 + e) + p.shift - 68)
+                     : (unsigned long long)sum[e];
         }
+#pragma unroll
+        for (int e = 0; e < 56; ++e) sum[e] = sum[e + 8];
         // turned in shared memory so that a warp writes four row pieces of 64
         // bytes at a time (per-row bulk reductions of 64 bytes from the staged
         // rows took 20 us a tile: the copy engine's rate of small operations)

@@ -276,7 +276,7 @@ static bool plan_limb_maps(stark_plan_s* p) {
 // share of its end, and the traffic of the divide (16 bytes written per
 // operand element), of the stored products and of the inputs and C at the
 // rates the passes reach (the deep F64 divides are bound by their fp64
-// additions, two a clock and SM).  Constants measured on GB300 at n = 200 to
+// additions, two a clock and SM).  Constants measured on GB300 at n = 130 to
 // 8192, depths 0 to 3; every pick there is within 6 % of the fastest depth.
 static double plan_seconds(int64_t n, int depth, stark_dtype dt) {
   const int64_t npad = padded_side(n, depth, dt), L = npad >> depth;
@@ -288,7 +288,8 @@ static double plan_seconds(int64_t n, int depth, stark_dtype dt) {
   cudaGetLastError();
   const double P = (double)pow7i(depth), side = std::ceil(L / 128.0), sms = have ? (double)v : 152.0;
   const double rounds = std::ceil(P * side * side / sms), chunks = L / 128.0;
-  const double leaf = f64 ? rounds * (chunks * 16.0e-6 + 6e-6) + 40e-6 : rounds * (chunks * 14.8e-6 + 3e-6) + 19e-6;
+  const double leaf = f64 ? rounds * (chunks * 16.0e-6 + 4e-6) + (depth < 2 ? 38e-6 : 63e-6)
+                          : rounds * (chunks * 14.8e-6 + 3e-6) + (depth < 2 ? 19e-6 : 25e-6);
   const double bytes = P * L * L * (depth ? 48.0 : 32.0) + (double)n * n * (f64 ? 40.0 : 24.0);
   const double rate = f64 ? (depth <= 1 ? 5.0e12 : depth == 2 ? 3.3e12 : 2.2e12) : (depth <= 1 ? 6.0e12 : 4.6e12);
   return leaf + bytes / rate;

@@ -40,7 +40,17 @@ template <>
 struct AccOf<SmallI64> {
   using type = int;
 };
+// An fp64 input already turned to an integer (the sums of Emitter's leaves are
+// then integer sums, scaled to each leaf's exponent by a shift).
+struct FixedF64 {
+  double v;
+};
+template <>
+struct AccOf<FixedF64> {
+  using type = unsigned long long;
+};
 __device__ __forceinline__ SmallI64 load_one(const SmallI64* p) { return SmallI64{__ldcs(&p->v)}; }
+__device__ __forceinline__ FixedF64 load_one(const FixedF64* p) { return FixedF64{__ldcs(&p->v)}; }
 template <typename T>
 __device__ __forceinline__ T load_one(const T* p) {
   return __ldcs(p);
@@ -131,6 +141,7 @@ struct Emitter {
   const int32_t* exps = nullptr;  // of leaf 0's row (side 0) or first column (side 1)
   int64_t exp_leaf = 0;           // L
   int exp_step = 0;               // 0: one exponent for the vector, 1: one per column
+  int common[2] = {0, 0};         // FixedF64: exponents of the integer sums
   __half* mags = nullptr;         // null outside the first 128 of K
   int64_t mag_leaf = 0;           // 128 L
 
@@ -146,15 +157,18 @@ struct Emitter {
       for (int e = 0; e < 2; ++e) {
         if constexpr (std::is_same_v<Tin, double>)
           q[e] = fixed62(x.v[e], exps[(int64_t)leaf * exp_leaf + e * exp_step]);
+        else if constexpr (std::is_same_v<Tin, FixedF64>)  // (a zero operand row has zero sums)
+          q[e] = x.v[e] << ((common[e] - exps[(int64_t)leaf * exp_leaf + e * exp_step]) & 63);
         else
           q[e] = (unsigned long long)x.v[e];
         q[e] += 0x8080808080808080ull;
       }
+      constexpr bool kReal = std::is_same_v<Tin, double> || std::is_same_v<Tin, FixedF64>;
       const int64_t base = ((int64_t)leaf * 8 * plane_elems + offset) / 2;
       __half2* out = reinterpret_cast<__half2*>(hi) + base;
 #pragma unroll
       for (int d = 0; d < 8; ++d) {
-        const int byte = std::is_same_v<Tin, double> ? 7 - d : d;  // F64: most significant digit first
+        const int byte = kReal ? 7 - d : d;  // F64: most significant digit first
         const uint32_t w0 = (uint32_t)(q[0] >> (byte < 4 ? 0 : 32)), w1 = (uint32_t)(q[1] >> (byte < 4 ? 0 : 32));
         // bytes (w0.b, 0x64, w1.b, 0x64) of the pair
         const uint32_t sel = (uint32_t)(byte & 3) | ((uint32_t)(4 + (byte & 3)) << 4);
@@ -162,7 +176,7 @@ struct Emitter {
         const uint32_t h = __byte_perm(b, 0x64u, 0x4140u);
         const __half2 v = __hsub2(*reinterpret_cast<const __half2*>(&h), __half2half2(__ushort_as_half(0x6480)));
         __stcs(reinterpret_cast<unsigned int*>(out + d * (plane_elems / 2)), *reinterpret_cast<const unsigned int*>(&v));
-        if (d == 0 && std::is_same_v<Tin, double>) {
+        if (d == 0 && kReal) {
           if (mags) {
             const __half2 m = __habs2(v);
             *reinterpret_cast<__half2*>(mags + (int64_t)leaf * mag_leaf) = m;
@@ -279,7 +293,14 @@ struct Loader {
   int64_t n;    // rows and columns read; zeros beyond
   int64_t ld;   // row stride
   bool vec_ok;  // rows are VEC-aligned: vector loads allowed where in bounds
+  int common[2] = {0, 0};  // FixedF64: the columns' exponents
 
+  __device__ __forceinline__ Acc value(const Tin& x, int e) const {
+    if constexpr (std::is_same_v<Tin, FixedF64>)
+      return fixed62(x.v, common[e]);
+    else
+      return (Acc)x;
+  }
   __device__ __forceinline__ Vec<Acc, VEC> operator()(int64_t row, int64_t col) const {
     Vec<Acc, VEC> r;
     if (row < n && col + VEC <= n && vec_ok) {
@@ -291,15 +312,15 @@ struct Loader {
         for (int w = 0; w < W; ++w) raw[w] = __ldcs(reinterpret_cast<const int4*>(p) + w);
         const Tin* t = reinterpret_cast<const Tin*>(raw);
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) r.v[e] = (Acc)t[e];
+        for (int e = 0; e < VEC; ++e) r.v[e] = value(t[e], e);
       } else {
 #pragma unroll
-        for (int e = 0; e < VEC; ++e) r.v[e] = (Acc)load_one(p + e);
+        for (int e = 0; e < VEC; ++e) r.v[e] = value(load_one(p + e), e);
       }
     } else {
 #pragma unroll
       for (int e = 0; e < VEC; ++e)
-        r.v[e] = (row < n && col + e < n) ? (Acc)load_one(X + row * ld + col + e) : Acc(0);
+        r.v[e] = (row < n && col + e < n) ? value(load_one(X + row * ld + col + e), e) : Acc(0);
     }
     return r;
   }
@@ -399,9 +420,17 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
     ld.npad = a.npad << K;  // a.npad is the subproblem's side
   } else {
     ld = ld0;
+    if constexpr (std::is_same_v<Tin, FixedF64>) {
+      ld.common[0] = a.common[SIDE == 0 ? i : j];
+      ld.common[1] = a.common[SIDE == 0 ? i : j + 1];
+    }
   }
   Emitter<OUT, Tin, VEC> emit{a.out_hi, a.out_lo, a.L * a.L, i * a.L + j, a.range_flag};
-  if constexpr (OUT == kOutLimbs && std::is_same_v<Tin, double>) {
+  if constexpr (std::is_same_v<Tin, FixedF64>) {
+    emit.common[0] = ld.common[0];
+    emit.common[1] = ld.common[1];
+  }
+  if constexpr (OUT == kOutLimbs && !std::is_same_v<Tin, int64_t>) {
     emit.exps = a.exps + (SIDE == 0 ? i : j);
     emit.exp_leaf = a.L;
     emit.exp_step = SIDE;
@@ -414,6 +443,21 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
   }
   const int64_t npad = a.npad;
 
+  auto run_tree = [&](const Vec<Acc, VEC>(&in)[pow4c(R)], int prefix) {
+    if constexpr (OUT == kOutLimbs && R == 2) {
+      // the seven products of the first level by one copy of the code (all 49
+      // leaves unrolled are 100 KB of digits a side, fetched by every wave)
+#pragma unroll 1
+      for (int m = 0; m < 7; ++m) {
+        Vec<Acc, VEC> o[4];
+#pragma unroll
+        for (int h = 0; h < 4; ++h) o[h] = level_sum<SIDE, Vec<Acc, VEC>>(m, [&](int q) { return in[q * 4 + h]; });
+        Tree<Acc, SIDE, 1, VEC>::run(o, prefix * 7 + m, emit);
+      }
+    } else {
+      Tree<Acc, SIDE, R, VEC>::run(in, prefix, emit);
+    }
+  };
   auto leaf_block = [&](const int* dig, int prefix) {
     // the 4^R sub-quadrant vectors below this prefix, then the register tree
     Vec<Acc, VEC> in[pow4c(R)];
@@ -441,7 +485,7 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
           in[g] = t.sb > 0 ? in[g] + w : in[g] - w;
         }
       }
-      Tree<Acc, SIDE, R, VEC>::run(in, prefix, emit);
+      run_tree(in, prefix);
       return;
     }
 #pragma unroll
@@ -455,7 +499,7 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
       }
       in[g] = Prefix<SIDE, Acc, VEC, F, LoadT>::eval(ld, dig, npad, r, c);
     }
-    Tree<Acc, SIDE, R, VEC>::run(in, prefix, emit);
+    run_tree(in, prefix);
   };
 
   if constexpr (F == 0) {

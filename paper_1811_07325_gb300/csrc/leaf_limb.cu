@@ -5,7 +5,8 @@
 // 1.25 TFLOP/s; the tensor cores run fp16 products three orders of magnitude
 // faster.  A digit in [-128, 127] is exact in fp16, a product of two at most
 // 2^14, and a sum of up to 1024 such products exact in the fp32 accumulator,
-// so a digit GEMM over K <= 128 with at most eight products per k is exact
+// so a digit GEMM over K <= 128 with at most eight products per k (or K <= 256
+// with four) is exact
 // integer arithmetic.  With x = sum_i x_i 256^i and y likewise,
 //   I64  x y mod 2^64 = sum_{s <= 7} 256^s D_s,      D_s = sum_{i+j=s} x_i y_j
 // (the divide writes plane i = digit i, least significant first), and
@@ -22,17 +23,18 @@
 //   warps 4..11 epilogue: two warps per TMEM lane quarter, 64 columns each
 //               (two warpgroups with 208 registers a thread, the first one
 //               keeps 88; 128 x 88 + 256 x 208 are the 384 x 168 of the launch).
-//               Every 128 of K the eight diagonals are drained from TMEM,
-//               converted to int32 (exact) and added into a 64-bit running
-//               sum held in registers; after the last superchunk the sums
+//               Each phase's diagonals are drained from TMEM, converted to
+//               int32 (exact) and added into a 64-bit running sum held in
+//               registers; after the last superchunk the sums
 //               (F64: rescaled and rounded once) are added into the leaf's C
 //               targets by bulk reductions.
 //
-// Order of the products.  TMEM holds four 128 x 128 accumulators, so a
-// superchunk (128 of K) runs in two phases: diagonals 7, 6, 5, 4 on
-// accumulators 0, 1, 2, 3 over all digits (26 products; quads A0-3, B0-3,
-// B4-7, A4-7 of each K block), then 3, 2, 1, 0 on accumulators 3, 2, 1, 0 over
-// the low four digits (10 products).  A block of 32 of K costs 72 MMAs for
+// Order of the products.  TMEM holds four 128 x 128 accumulators, so K runs in
+// superchunks of 256 with three phases: twice, for each 128 of K, diagonals
+// 7, 6, 5, 4 on accumulators 0, 1, 2, 3 over all digits (26 products a block;
+// quads A0-3, B0-3, B4-7, A4-7 of each K block), then for all 256 diagonals
+// 3, 2, 1, 0 on accumulators 3, 2, 1, 0 over the low four digits (10 products,
+// at most four per diagonal, so exact over twice the K).  A block of 32 of K costs 72 MMAs for
 // 192 KB of operands.  Each phase ends its accumulators one after another in
 // the order in which the other phase starts on them, so that the epilogue
 // drains one while the tensor cores fill the others.  All of this order is
@@ -118,7 +120,7 @@ __global__ void __launch_bounds__(kThreadsL, 1)
   const int per_leaf = tiles * tiles;
   const int num_items = (p.leaf_end - p.leaf_begin) * per_leaf;
   const int kblocks = p.L / 32;         // even
-  const int chunks = (kblocks + 3) / 4;  // superchunks of four blocks, the last one possibly of two
+  const int chunks = (kblocks + 3) / 4;  // 128 of K each, the last one possibly 64
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kQuads; ++s) {
@@ -202,16 +204,11 @@ __global__ void __launch_bounds__(kThreadsL, 1)
           }
         }
         const int plane = leaf * kDigits;
-        for (int c = 0; ok && c < chunks; ++c) {
-          const int k0 = c * 128, blocks = kblocks - 4 * c < 4 ? kblocks - 4 * c : 4;
-          for (int b = 0; ok && b < blocks; ++b) {
-            const int k = k0 + b * 32;
+        for (int k0 = 0; ok && k0 < p.L; k0 += 256) {
+          const int k1 = k0 + 256 < p.L ? k0 + 256 : p.L;
+          for (int k = k0; ok && k < k1; k += 32)
             ok = load_a(k, m0, plane) && load_b(k, n0, plane) && load_b(k, n0, plane + 4) && load_a(k, m0, plane + 4);
-          }
-          for (int b = 0; ok && b < blocks; ++b) {
-            const int k = k0 + b * 32;
-            ok = load_a(k, m0, plane) && load_b(k, n0, plane);
-          }
+          for (int k = k0; ok && k < k1; k += 32) ok = load_a(k, m0, plane) && load_b(k, n0, plane);
         }
       }
       if (!ok) {
@@ -258,9 +255,10 @@ __global__ void __launch_bounds__(kThreadsL, 1)
           mma_f16(tmem_base + (uint32_t)acc * 128u, da, db, IDESC, first && k == 0 ? 0u : 1u);
         }
       };
-      // diagonals 7..4 of a K block: by diagonal (the first block of a
-      // superchunk; it starts the accumulators in turn), or by quad (the
-      // others; quads are freed early and the last block ends 4, 5, 6, 7)
+      // diagonals 7..4 of a K block: by diagonal (the first block after a low
+      // phase; it starts the accumulators in the order that phase frees them),
+      // or by quad (the others; quads are freed early and the last block of a
+      // phase ends 4, 5, 6, 7)
       auto high_first = [&]() -> bool {
         int sa[2], sb[2];
         if ((sa[0] = take()) < 0 || (sb[0] = take()) < 0 || (sb[1] = take()) < 0 || (sa[1] = take()) < 0) return false;
@@ -285,7 +283,7 @@ __global__ void __launch_bounds__(kThreadsL, 1)
         mma_commit(empty_bar(sb[0]));
         return true;
       };
-      auto high_next = [&](bool last) -> bool {
+      auto high_next = [&](bool first, bool last) -> bool {
         int sa[2], sb[2];
         if ((sa[0] = take()) < 0 || (sb[0] = take()) < 0) return false;
         tc_fence_after();
@@ -293,14 +291,26 @@ __global__ void __launch_bounds__(kThreadsL, 1)
 #pragma unroll
         for (int s = 4; s <= 6; ++s)
 #pragma unroll
-          for (int i = s - 3; i <= 3; ++i) mul(a0, b0, i, s - i, 7 - s, false);
+          for (int i = s - 3; i <= 3; ++i) {
+            if (i == s - 3 && first) {
+              if (!wait_free(7 - s)) return false;
+              tc_fence_after();
+            }
+            mul(a0, b0, i, s - i, 7 - s, i == s - 3 && first);
+          }
         if ((sb[1] = take()) < 0) return false;
         tc_fence_after();
         const uint32_t b1 = lo_b(sb[1]);
 #pragma unroll
         for (int s = 4; s <= 7; ++s)
 #pragma unroll
-          for (int i = 0; i <= s - 4; ++i) mul(a0, b1, i, s - 4 - i, 7 - s, false);
+          for (int i = 0; i <= s - 4; ++i) {
+            if (s == 7 && i == 0 && first) {
+              if (!wait_free(0)) return false;
+              tc_fence_after();
+            }
+            mul(a0, b1, i, s - 4 - i, 7 - s, s == 7 && i == 0 && first);
+          }
         mma_commit(empty_bar(sa[0]));
         mma_commit(empty_bar(sb[1]));
         if ((sa[1] = take()) < 0) return false;
@@ -356,12 +366,12 @@ __global__ void __launch_bounds__(kThreadsL, 1)
       };
       for (int item = blockIdx.x; ok && item < num_items; item += gridDim.x) {
         if (F64) ok = check();
-        for (int c = 0; ok && c < chunks; ++c) {
-          const int blocks = kblocks - 4 * c < 4 ? kblocks - 4 * c : 4;  // 4 or 2
+        for (int b0 = 0; ok && b0 < kblocks; b0 += 8) {
+          const int b1 = b0 + 8 < kblocks ? b0 + 8 : kblocks;
           issued = true;
           ok = high_first();
-          for (int b = 1; ok && b < blocks; ++b) ok = high_next(b == blocks - 1);
-          for (int b = 0; ok && b < blocks; ++b) ok = low(b == 0, b == blocks - 1);
+          for (int b = b0 + 1; ok && b < b1; ++b) ok = high_next((b & 3) == 0, (b & 3) == 3 || b == b1 - 1);
+          for (int b = b0; ok && b < b1; ++b) ok = low(b == b0, b == b1 - 1);
         }
       }
       if (!ok && issued) {
@@ -468,7 +478,11 @@ __global__ void __launch_bounds__(kThreadsL, 1)
       for (int c = 0; ok && c < chunks; ++c) {
         // in the order in which the issuer finishes them: 4..7, then 0..3
 #pragma unroll 1
-        for (int x = 0; ok && x < 8; ++x) ok = x < 4 ? drain(3 - x, x + 4) : drain(x - 4, x - 4);
+        for (int x = 0; ok && x < 4; ++x) ok = drain(3 - x, x + 4);
+        if ((c & 1) || c == chunks - 1) {
+#pragma unroll 1
+          for (int x = 0; ok && x < 4; ++x) ok = drain(x, x);
+        }
       }
       if (!ok) break;
       // combine: the row segment goes into every C target of the leaf

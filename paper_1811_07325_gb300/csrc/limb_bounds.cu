@@ -79,10 +79,34 @@ __global__ void __launch_bounds__(256) limb_max_kernel(LimbBoundsArgs a) {
 // One thread per (leaf, row of A) and (leaf, column of B).  Per depth, so that
 // the terms sit in registers and their loads are in flight together (33 us at
 // n = 1024, depth 3, with a loop over a local array).
+// Grid y 2 and 3: the common exponents.  A row position i of the L x L leaf
+// grid sees 4^D input quadrants; where their largest magnitudes (zeros aside)
+// lie within a factor of four, all are turned to integers by one exponent
+// ec = e(largest) + D, the operand sums are integer sums, and a leaf's digits
+// are the sum shifted by ec - e(leaf): off by at most 2^(D + 2) of the 2^-62 R
+// units per term, still 2^-57 R, where an fp64 sum is rounded to 2^-53.
 template <int D>
 __global__ void __launch_bounds__(256) limb_exp_kernel(LimbBoundsArgs a, int64_t leaves) {
   const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
-  const int side = blockIdx.y;
+  const int side = blockIdx.y & 1;
+  if (blockIdx.y >= 2) {
+    if (t >= a.L) return;
+    const double* mq = side == 0 ? a.max_a : a.max_b;
+    unsigned long long mx = 0, mn = ~0ull;
+    for (int q = 0; q < (1 << D); ++q)  // blocks along K, then along the rows of A (columns of B)
+#pragma unroll
+      for (int r = 0; r < (1 << D); ++r) {
+        const unsigned long long b = mag_bits(mq[q * a.npad + r * a.L + t]);
+        mx = max(mx, b);
+        if (b != 0) mn = min(mn, b);
+      }
+    const int ex = (int)(mx >> 52);
+    int32_t ec = mx == 0 ? 0 : ex - 1023 + ((mx & 0xFFFFFFFFFFFFFull) ? 1 : 0) + D;
+    // (magnitude bits: two exponents apart is a factor of four)
+    if (mx != 0 && (ex == 2047 || ex < 8 || mn + (2ull << 52) < mx)) ec = kLimbZeroRow;
+    (side == 0 ? a.common_a : a.common_b)[t] = ec;
+    return;
+  }
   if (t >= leaves * a.L) return;
   const int leaf = (int)(t / a.L);
   const int64_t i = t % a.L;  // row (side 0) or column (side 1) of the leaf
@@ -131,7 +155,7 @@ __global__ void __launch_bounds__(256) limb_exp_kernel(LimbBoundsArgs a, int64_t
 
 template <int D>
 void launch_exp(const LimbBoundsArgs& a, int64_t leaves, cudaStream_t st) {
-  limb_exp_kernel<D><<<dim3((unsigned)((leaves * a.L + 255) / 256), 2), 256, 0, st>>>(a, leaves);
+  limb_exp_kernel<D><<<dim3((unsigned)((leaves * a.L + 255) / 256), 4), 256, 0, st>>>(a, leaves);
 }
 
 }  // namespace

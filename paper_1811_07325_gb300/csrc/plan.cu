@@ -924,7 +924,8 @@ static bool plan_limb_alloc(stark_plan_s* p, int64_t ws) {
     const int64_t maxima = (p->npad << p->depth) * 8, exps = (p->P * p->L * 4 + 255) / 256 * 256,
                   mags = p->P * p->L * kLimbCheckK * 2;
     const int64_t needs = (p->P * 4 + 255) / 256 * 256;
-    aux = 256 + needs + 2 * (maxima + exps + mags);
+    const int64_t commons = (p->L * 4 + 255) / 256 * 256;
+    aux = 256 + needs + 2 * (maxima + exps + mags + commons);
     ok = cudaMalloc(&p->limb_aux, (size_t)aux) == cudaSuccess;
     if (ok) {
       char* b = static_cast<char*>(p->limb_aux);
@@ -932,6 +933,9 @@ static bool plan_limb_alloc(stark_plan_s* p, int64_t ws) {
       b += 256;  // every part is a multiple of 256 bytes
       p->limb_need = reinterpret_cast<float*>(b);
       b += needs;
+      p->common_a = reinterpret_cast<int32_t*>(b);
+      p->common_b = reinterpret_cast<int32_t*>(b + commons);
+      b += 2 * commons;
       p->mag_a = b;
       p->mag_b = b + mags;
       b += 2 * mags;
@@ -1384,10 +1388,13 @@ static stark_status plan_limb_divide(stark_plan_s* p, const void* A, const void*
   DivideArgs db{B, core_side(p), p->npad, p->L, p->Y, nullptr, p->d_err, -1, p->n};
   if (p->dt == STARK_F64) {
     const LimbBoundsArgs b{static_cast<const double*>(A), static_cast<const double*>(B), core_side(p), p->n, p->npad,
-                           p->L, p->depth, p->max_a, p->max_b, p->exp_a, p->exp_b, p->d_flag};
+                           p->L, p->depth, p->max_a, p->max_b, p->exp_a, p->exp_b, p->common_a, p->common_b,
+                           p->d_flag};
     if (stark_status st = to_status(launch_limb_bounds(b, s)); st != STARK_OK) return st;
     da.exps = p->exp_a;
     db.exps = p->exp_b;
+    da.common = p->common_a;
+    db.common = p->common_b;
     da.mags = p->mag_a;
     db.mags = p->mag_b;
   }

@@ -91,6 +91,8 @@ struct stark_plan_s {
   double* max_b = nullptr;   // and of B's columns
   int32_t* exp_a = nullptr;  // [P][L] exponents of the leaf operands' rows
   int32_t* exp_b = nullptr;  // and columns
+  int32_t* common_a = nullptr;  // [L] exponents shared by the leaves (limb_bounds.cu)
+  int32_t* common_b = nullptr;
   void* mag_a = nullptr;     // [P][L][128] magnitudes of the leading digits
   void* mag_b = nullptr;     // [P][128][L]
   float* limb_need = nullptr;  // [P] magnitude sums that prove a leaf's elements

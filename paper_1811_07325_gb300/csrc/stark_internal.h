@@ -84,6 +84,9 @@ struct DivideArgs {
   // or columns (side 1), and the digit-magnitude planes of the first 128 of K
   // ([leaf][L][128] for side 0, [leaf][128][L] for side 1)
   const int32_t* exps;
+  // exponents [L] that all the leaves' rows (columns) at one position share, or
+  // kLimbZeroRow where they differ too much (limb_bounds.cu)
+  const int32_t* common;
   void* mags;
 };
 
@@ -117,6 +120,8 @@ struct LimbBoundsArgs {
   double* max_b;      // [2^depth row blocks][npad]: column maxima of |B|
   int32_t* expA;      // [7^depth][L]
   int32_t* expB;
+  int32_t* common_a;  // [L]
+  int32_t* common_b;
   int* flag;          // cleared, then set for infinities, NaN and exponents outside +-400
 };
 cudaError_t launch_limb_bounds(const LimbBoundsArgs& a, cudaStream_t s);

@@ -134,6 +134,29 @@ def test_f64_unproven_products_are_redone(stark_lib):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("scale", [2.0 ** -1, 2.0 ** -30])
+@pytest.mark.parametrize("d", [1, 2])
+def test_f64_row_blocks_of_different_scale(stark_lib, d, scale):
+    # rows of the lower half (columns of B's left half) scaled: by one half the
+    # quadrants share an exponent and the operand sums are integer sums, by
+    # 2^-30 they do not; C21 has products of the scaled blocks only, and is
+    # accurate at its own scale
+    S = stark_lib
+    n = 512
+    A, B = synth.uniform(n, 35, 0), synth.normal(n, 35, 1).astype(np.float64)
+    A[n // 2:] *= scale
+    B[:, : n // 2] *= scale
+    want = oracle.gemm_classical(A, B)
+    with S.Plan(n, d, S.DType.F64) as p:
+        C = p.mul(dev(A), dev(B)).cpu().numpy()
+        p.check()
+        L = p.leaf
+    assert np.abs(C - want).max() <= strassen_bound(n, d, L, A, B)
+    h = slice(n // 2, n), slice(0, n // 2)
+    assert np.abs(C - want)[h].max() <= strassen_bound(n, d, L, A[h[0]], B[:, h[1]])
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("dtype,n,d,peel", [("I64", 600, 1, False), ("F64", 600, 1, False), ("I64", 650, 2, True),
                                             ("F64", 650, 2, True)])
 def test_limb_leaf_ranges_traversal_and_capture(stark_lib, dtype, n, d, peel):

@@ -10,7 +10,7 @@
 //
 // Depth per member: given, or chosen by the autotuner, which times the
 // candidate (depth, leaf tile) pairs on the device (one warm-up and three
-// timed products per candidate on scratch inputs) and caches the winner per
+// rounds of two timed products per candidate on scratch inputs) and caches the winner per
 // size class and dtype for the process.  The tile candidates are CTA pairs
 // on 256 x 256 tiles (cta_group::2; leaf sides that are multiples of 256)
 // and single CTAs on 128 x 128 tiles.  Members whose tile is 256 share up to
@@ -20,6 +20,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <tuple>
 #include <vector>
 
 #include "plan.h"
@@ -29,12 +30,16 @@ namespace stark {
 namespace {
 
 std::mutex g_tune_mu;
-std::map<std::pair<int64_t, int>, std::pair<int, int>> g_tuned;  // (n class, dtype) -> (depth, tile)
+// (n class, dtype, grouped) -> (depth, tile)
+std::map<std::tuple<int64_t, int, bool>, std::pair<int, int>> g_tuned;
 
 // Device time (ms) of one product of side n at `depth` with leaf tiles of
-// width `tile` (256: CTA pairs; 128: single CTAs), averaged over 3.
-float time_depth(int64_t n, int depth, stark_dtype dt, int tile, void* A, void* B, void* C, cudaStream_t s) {
+// width `tile` (256: CTA pairs; 128: single CTAs), the best of three rounds; grouped:
+// without K slices, which a member of a grouped launch does not get.
+float time_depth(int64_t n, int depth, stark_dtype dt, int tile, bool grouped, void* A, void* B, void* C,
+                 cudaStream_t s) {
   stark_plan_s p;
+  p.whole_k = grouped;
   if (plan_init(&p, n, depth, dt) != STARK_OK) {
     plan_release(&p);
     return -1.f;
@@ -51,11 +56,16 @@ float time_depth(int64_t n, int depth, stark_dtype dt, int tile, void* A, void* 
   cudaEventCreate(&e1);
   float ms = -1.f;
   if (plan_run(&p, A, B, C, 0, p.P, s) == STARK_OK) {
-    cudaEventRecord(e0, s);
     bool ok = true;
-    for (int r = 0; r < 3 && ok; ++r) ok = plan_run(&p, A, B, C, 0, p.P, s) == STARK_OK;
-    cudaEventRecord(e1, s);
-    if (ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess) ms /= 3;
+    for (int round = 0; round < 3 && ok; ++round) {  // the best of three rounds of two
+      cudaEventRecord(e0, s);
+      for (int r = 0; r < 2 && ok; ++r) ok = plan_run(&p, A, B, C, 0, p.P, s) == STARK_OK;
+      cudaEventRecord(e1, s);
+      float t = 0;
+      if (ok && cudaEventSynchronize(e1) == cudaSuccess && cudaEventElapsedTime(&t, e0, e1) == cudaSuccess && t > 0 &&
+          (ms < 0 || t / 2 < ms))
+        ms = t / 2;
+    }
   }
   cudaStreamSynchronize(s);
   cudaEventDestroy(e0);
@@ -68,13 +78,15 @@ float time_depth(int64_t n, int depth, stark_dtype dt, int tile, void* A, void* 
 }  // namespace
 
 // Measured depth choice for n x n products (cached per process).
-void autotune(int64_t n_req, stark_dtype dt, int* depth_out, int* tile_out) {
+// A level of recursion doubles the error, so a deeper candidate has to be
+// faster by 4 % (the spread of these short timings) to be taken.
+void autotune(int64_t n_req, stark_dtype dt, bool grouped, int* depth_out, int* tile_out) {
   // size class: n rounded up to 64 (n <= 1024), 128 (n <= 2048), else 256
   const int64_t q = n_req <= 1024 ? 64 : n_req <= 2048 ? 128 : 256;
   const int64_t n = (n_req + q - 1) / q * q;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tuned.find({n, (int)dt});
+    auto it = g_tuned.find({n, (int)dt, grouped});
     if (it != g_tuned.end()) {
       *depth_out = it->second.first;
       *tile_out = it->second.second;
@@ -91,14 +103,16 @@ void autotune(int64_t n_req, stark_dtype dt, int* depth_out, int* tile_out) {
     cudaMemsetAsync(A, 0x3c, bytes, s);  // bounded, nonzero values
     cudaMemsetAsync(B, 0x3c, bytes, s);
     float best_ms = 1e30f;
+    int best_d = 0;
     for (int d = 0; d <= 3; ++d) {
       if ((padded_side(n, d, dt) >> d) < tile_granularity(dt)) continue;
       if (d > 0 && (n >> d) < 128) break;
       const bool wide = (padded_side(n, d, dt) >> d) % 256 == 0;
       for (int tile : {256, 128}) {
         if (tile == 256 && !wide) continue;
-        const float ms = time_depth(n, d, dt, tile, A, B, C, s);
-        if (ms > 0 && ms < best_ms) {
+        const float ms = time_depth(n, d, dt, tile, grouped, A, B, C, s);
+        if (ms > 0 && ms < best_ms * (d > best_d ? 0.96f : 1.f)) {
+          best_d = d;
           best_ms = ms;
           best = d;
           best_tile = tile;
@@ -112,14 +126,14 @@ void autotune(int64_t n_req, stark_dtype dt, int* depth_out, int* tile_out) {
   cudaFree(C);
   cudaGetLastError();
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tuned[{n, (int)dt}] = {best, best_tile};
+  g_tuned[{n, (int)dt, grouped}] = {best, best_tile};
   *depth_out = best;
   *tile_out = best_tile;
 }
 
-int autotune_depth(int64_t n, stark_dtype dt) {
+int autotune_depth(int64_t n, stark_dtype dt, bool grouped) {
   int d = 0, tile = 128;
-  autotune(n, dt, &d, &tile);
+  autotune(n, dt, grouped, &d, &tile);
   return d;
 }
 
@@ -199,7 +213,7 @@ stark_status stark_batch_create(int32_t count, const int64_t* n, int depth, star
   b->tiles.assign(count, 128);
   for (int i = 0; i < count && st == STARK_OK; ++i) {
     int d = depth, tile = 0;
-    if (depth < 0) autotune(n[i], dt, &d, &tile);
+    if (depth < 0) autotune(n[i], dt, true, &d, &tile);
     auto* p = new (std::nothrow) stark_plan_s();
     if (!p) {
       st = STARK_ENOMEM;

@@ -13,6 +13,8 @@ template <int OUT, int D>
 __global__ void __launch_bounds__(256, 2)
     divide_pair_kernel(DivideArgs a, DivideArgs b, int vec_a, int vec_b, float* zero, int64_t zero_count) {
   grid_launch_dependents();
+  // (the clear goes last, its lines are still in L2 when the leaf kernel adds:
+  // first, 3xTF32 at n = 4096, depth 2 took 542 instead of 531 us)
   if (blockIdx.z == 0) {
     divide_body<float, OUT, D, 0, 4, 0>(a, vec_a);
   } else if (blockIdx.z == 1) {

@@ -42,9 +42,11 @@
 // steps, the issuing thread needed 760 cycles a step on its own and the
 // kernel ran at 30 % of the fp16 rate (6.5 ms for 49 leaves of side 1024).
 //
-// F64 accuracy.  The integers x_i keep 62 bits below the row's bound R (a
-// power of two), and with C the bound of the column of B a product of K
-// non-zero terms is off by at most K 2^-59 R C (the dropped digit products,
+// F64 accuracy.  The operands are sums of up to 2^d inputs: an fp64 sum rounded
+// to 2^-62 of the row's bound R (a power of two), or an integer sum off by at
+// most 2^(d+2) such units (limb_bounds.cu), 2^-57 R at depth 3, where the fp64
+// sums alone are off by 2^-53 of themselves a level.  Given them, and with C
+// the bound of the column of B, a product of K non-zero terms is off by at most K 2^-59 R C (the dropped digit products,
 // 7 * 2^14 * 256^6 / 2^124 a term) and three half units of the running sum
 // per superchunk, the unit being L 2^-62 R C.  A K-term FP64 dot product is
 // only bound to K 2^-53 sum |a||b|.  So the digits are the more accurate of

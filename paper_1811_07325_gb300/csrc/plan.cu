@@ -644,9 +644,8 @@ static stark_status plan_tune_combine(stark_plan_t p) {
 }
 
 // Workspace for `planes_per_half` leaves per operand side, with its maps.
-static stark_status plan_alloc_operands(stark_plan_s* p, int64_t planes) {
-  // bytes per leaf element per operand (digit planes: only breadth first)
-  const int64_t per = half_split(p->dt) ? 4 : p->limb_ok && planes == p->P ? 16 : 8;
+// (per: bytes per leaf element and operand).
+static stark_status plan_alloc_operands_at(stark_plan_s* p, int64_t planes, int64_t per) {
   const int64_t bytes = planes * p->L * p->L * per;
   if (cudaDeviceSynchronize() != cudaSuccess) return STARK_ECUDA;
   const int64_t old = p->P_ws * p->L * p->L * p->op_elem;
@@ -688,6 +687,14 @@ static stark_status plan_alloc_operands(stark_plan_s* p, int64_t planes) {
                     !make_tmap_planes(&p->tmBi, p->Y, false, p->L, planes, 64)))
     return STARK_EUNSUPPORTED;
   return STARK_OK;
+}
+
+static stark_status plan_alloc_operands(stark_plan_s* p, int64_t planes) {
+  if (p->limb_ok && planes == p->P) {  // digit planes, where they fit (breadth first only)
+    const stark_status st = plan_alloc_operands_at(p, planes, 16);
+    if (st != STARK_ENOMEM) return st;
+  }
+  return plan_alloc_operands_at(p, planes, half_split(p->dt) ? 4 : 8);
 }
 
 stark_status stark_plan_set_traversal(stark_plan_t p, int levels) {
@@ -1231,7 +1238,7 @@ static bool plan_tma_c(const stark_plan_s* p, const void* C) {
 // again, its slices adding into C like tiles of other leaves.  n = 256 has one
 // tile of 256 x 256; whole it took 12.4 us of leaf kernel.
 static int plan_ksplit(const stark_plan_s* p, const void* C, int64_t lb, int64_t le) {
-  if (!plan_tma_c(p, C) || p->promo_k || p->deep_pipeline || p->dfs || p->shard_levels) return 1;
+  if (p->whole_k || !plan_tma_c(p, C) || p->promo_k || p->deep_pipeline || p->dfs || p->shard_levels) return 1;
   const bool wide = p->pair_mode == 2 && p->bn == 256;
   const int64_t tm = p->L / (wide ? 256 : 128), tn = p->L / p->bn;
   const int64_t items = (le - lb) * tm * tn, units = wide ? p->num_sms / 2 : p->num_sms;
@@ -1278,7 +1285,10 @@ static stark_status plan_leaves(stark_plan_s* p, void* C, int64_t lb, int64_t le
       a.ksplit = plan_ksplit(p, C, lb, le);
       if (plan_direct(p, C, lb, le)) a.use_tma_c = 2;
     }
-    a.pdl = !p->dfs && !p->shard_levels && p->depth <= 2 ? 1 : 0;  // after launch_divide_pair
+    // the leaf kernel's prologue under the divide (launch_divide_pair) of small
+    // products (n = 4096, depth 2: 539 for 541 us); at n = 16384 it cost 1 %
+    // (the waiting CTAs sit beside the divide's last blocks)
+    a.pdl = !p->dfs && !p->shard_levels && p->depth <= 2 && p->P * p->L * p->L <= (int64_t)1 << 26 ? 1 : 0;
     if (deterministic) {
       a.store_m = 1;
       a.use_tma_c = 0;

@@ -1,5 +1,5 @@
 // divide_pair.cu -- the split-fp32 divide of both operands at depth <= 2 in
-// one launch, which also clears C (or its staging copy) where the combine adds
+// one launch (two at depth 2), which also clears C (or its staging copy) where the combine adds
 // into it: grid z is A, B, clear.  For small products the phases before the
 // leaf kernel are launches, not bytes: cleared and divided by a memset and two
 // kernels, n = 256 spent 16 of its 27 us there.  The leaf kernel that follows
@@ -9,15 +9,20 @@
 namespace stark {
 namespace {
 
-template <int OUT, int D>
+// SIDES 0: A (and the clear after it), 1: B (the same), 2: both.  Depth 2 runs
+// A and B in turn: its code is unrolled over 49 planes, and blocks of both sides
+// on one SM fetched it past each other (3xTF32 at n = 1536 34.8 us in turn, 46.4
+// together; 3xFP16 at n = 1694 29.3 and 38.4).  Depths 0 and 1 are faster
+// together (3xTF32 at n = 1536, depth 1: 23.0 in turn, 17.9).
+template <int OUT, int D, int SIDES>
 __global__ void __launch_bounds__(256, 2)
     divide_pair_kernel(DivideArgs a, DivideArgs b, int vec_a, int vec_b, float* zero, int64_t zero_count) {
   grid_launch_dependents();
   // (the clear goes last, its lines are still in L2 when the leaf kernel adds:
   // first, 3xTF32 at n = 4096, depth 2 took 542 instead of 531 us)
-  if (blockIdx.z == 0) {
+  if (SIDES != 1 && blockIdx.z == 0) {
     divide_body<float, OUT, D, 0, 4, 0>(a, vec_a);
-  } else if (blockIdx.z == 1) {
+  } else if (SIDES != 0 && blockIdx.z == (SIDES == 1 ? 0 : 1)) {
     divide_body<float, OUT, D, 1, 4, 0>(b, vec_b);
   } else {
     const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x, step = (int64_t)gridDim.x * 256;
@@ -33,10 +38,18 @@ cudaError_t launch(const DivideArgs& a, const DivideArgs& b, void* zero, int64_t
   auto vec = [](const DivideArgs& x) { return x.ld % 4 == 0 && (reinterpret_cast<uintptr_t>(x.X) & 15) == 0 ? 1 : 0; };
   const int64_t blocks = (a.L * (a.L / 4) + 255) / 256;
   if (blocks > 0x7FFFFFFF) return cudaErrorInvalidValue;
-  divide_pair_kernel<OUT, D><<<dim3((unsigned)blocks, 1, zero ? 3 : 2), 256, 0, st>>>(
-      a, b, vec(a), vec(b), static_cast<float*>(zero), zero_bytes / 4);
-  count_launch();
-  return cudaGetLastError();
+  const auto go = [&](auto kernel, int parts, void* clear) {
+    kernel<<<dim3((unsigned)blocks, 1, clear ? parts + 1 : parts), 256, 0, st>>>(
+        a, b, vec(a), vec(b), static_cast<float*>(clear), zero_bytes / 4);
+    count_launch();
+    return cudaGetLastError();
+  };
+  if constexpr (D < 2) {
+    return go(divide_pair_kernel<OUT, D, 2>, 2, zero);
+  } else {
+    const cudaError_t e = go(divide_pair_kernel<OUT, D, 0>, 1, nullptr);
+    return e == cudaSuccess ? go(divide_pair_kernel<OUT, D, 1>, 1, zero) : e;
+  }
 }
 
 template <int OUT>

@@ -102,9 +102,9 @@ typedef struct {
  * Alg. 2: depth = log2 of the number of partitions per side, the paper's
  * p - q).  depth = -1 lets the library choose: for the tensor-core dtypes a
  * measured autotuner times the candidate depths on the device once per size
- * class (n rounded up to 64, 128 or 256) and caches the winner for the process (the
- * paper's U-shaped optimum over the partition count, Sec. V-C, found by
- * measurement); for F64/I64 a cost model over leaf work and divide traffic.
+ * class (n rounded up to 64, 128 or 256) and caches, for the process, the most
+ * accurate one within 10 % of the fastest (the paper's U-shaped optimum over the
+ * partition count, Sec. V-C, found by measurement); for F64/I64 a cost model over leaf work and divide traffic.
  * depth 0 multiplies classically (one leaf).
  * Allocates the plan's device workspace on the current device.
  * Errors: EINVAL (n < 0 or > 2^20, depth < -1 or > 4, unknown dtype, out == NULL),
@@ -404,7 +404,7 @@ STARK_API stark_status stark_batch_mul(stark_batch_t batch, const void *const *A
 /* Leaf tile width of member `index` (caller's order): 256 (CTA pairs on
  * 256 x 256 tiles) or 128 (single CTAs on 128 x 128 tiles); with depth -1
  * the autotuner times both where the leaf side allows 256 and keeps the
- * faster (with its depth). */
+ * faster (at the depth it takes). */
 STARK_API stark_status stark_batch_tile(stark_batch_t batch, int32_t index, int32_t *tile_n);
 
 /* Depth chosen for member `index`. */

@@ -16,6 +16,7 @@
 // and single CTAs on 128 x 128 tiles.  Members whose tile is 256 share up to
 // three grouped launches of CTA pairs, the others one of single CTAs.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -30,14 +31,25 @@ namespace stark {
 namespace {
 
 std::mutex g_tune_mu;
-// (n class, dtype, grouped) -> (depth, tile)
-std::map<std::tuple<int64_t, int, bool>, std::pair<int, int>> g_tuned;
+// (n class, dtype) -> (depth, tile)
+std::map<std::pair<int64_t, int>, std::pair<int, int>> g_tuned;
+
+// Relative RMS error of a product of N(0, 1) inputs, as measured: the split's,
+// doubled by every level, and the tensor cores' accumulation, in proportion to
+// the K that one accumulation spans.
+double relative_error(const stark_plan_s& p, const void* C) {
+  const double k = (double)p.L / plan_k_slices(&p, C);
+  const double split = (p.dt == STARK_F32_SPLIT_BF16 ? 4.4e-6 : 1e-7) * (double)(1 << p.depth);
+  const double sums = (p.dt == STARK_F32_SPLIT_TF32 ? 7.0e-9 : p.dt == STARK_F32_SPLIT_FP16 ? 3.6e-9 : 3.4e-9) * k;
+  return std::sqrt(split * split + sums * sums);
+}
 
 // Device time (ms) of one product of side n at `depth` with leaf tiles of
 // width `tile` (256: CTA pairs; 128: single CTAs), the best of three rounds; grouped:
-// without K slices, which a member of a grouped launch does not get.
+// without K slices and narrow tiles, which a member of a grouped launch does
+// not get.
 float time_depth(int64_t n, int depth, stark_dtype dt, int tile, bool grouped, void* A, void* B, void* C,
-                 cudaStream_t s) {
+                 cudaStream_t s, double* error) {
   stark_plan_s p;
   p.whole_k = grouped;
   if (plan_init(&p, n, depth, dt) != STARK_OK) {
@@ -51,6 +63,7 @@ float time_depth(int64_t n, int depth, stark_dtype dt, int tile, bool grouped, v
     plan_release(&p);
     return -1.f;
   }
+  *error = relative_error(p, C);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -77,16 +90,16 @@ float time_depth(int64_t n, int depth, stark_dtype dt, int tile, bool grouped, v
 
 }  // namespace
 
-// Measured depth choice for n x n products (cached per process).
-// A level of recursion doubles the error, so a deeper candidate has to be
-// faster by 4 % (the spread of these short timings) to be taken.
-void autotune(int64_t n_req, stark_dtype dt, bool grouped, int* depth_out, int* tile_out) {
+// Measured depth choice for n x n products (cached per process): one for a plan,
+// a batch's member and a request, whose results then agree, by the time of the
+// product as a plan plus its time as a member.
+void autotune(int64_t n_req, stark_dtype dt, int* depth_out, int* tile_out) {
   // size class: n rounded up to 64 (n <= 1024), 128 (n <= 2048), else 256
   const int64_t q = n_req <= 1024 ? 64 : n_req <= 2048 ? 128 : 256;
   const int64_t n = (n_req + q - 1) / q * q;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
-    auto it = g_tuned.find({n, (int)dt, grouped});
+    auto it = g_tuned.find({n, (int)dt});
     if (it != g_tuned.end()) {
       *depth_out = it->second.first;
       *tile_out = it->second.second;
@@ -102,22 +115,41 @@ void autotune(int64_t n_req, stark_dtype dt, bool grouped, int* depth_out, int* 
       cudaMalloc(&C, bytes) == cudaSuccess && cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking) == cudaSuccess) {
     cudaMemsetAsync(A, 0x3c, bytes, s);  // bounded, nonzero values
     cudaMemsetAsync(B, 0x3c, bytes, s);
+    struct Candidate {
+      int depth, tile;
+      float ms;
+      double error;
+    };
+    std::vector<Candidate> tried;
     float best_ms = 1e30f;
-    int best_d = 0;
     for (int d = 0; d <= 3; ++d) {
       if ((padded_side(n, d, dt) >> d) < tile_granularity(dt)) continue;
       if (d > 0 && (n >> d) < 128) break;
       const bool wide = (padded_side(n, d, dt) >> d) % 256 == 0;
+      double plan_error;
+      const float plan_ms = time_depth(n, d, dt, wide ? 256 : 128, false, A, B, C, s, &plan_error);
       for (int tile : {256, 128}) {
         if (tile == 256 && !wide) continue;
-        const float ms = time_depth(n, d, dt, tile, grouped, A, B, C, s);
-        if (ms > 0 && ms < best_ms * (d > best_d ? 0.96f : 1.f)) {
-          best_d = d;
-          best_ms = ms;
-          best = d;
-          best_tile = tile;
+        Candidate c{d, tile, 0.f, 0.0};
+        c.ms = time_depth(n, d, dt, tile, true, A, B, C, s, &c.error);
+        if (c.ms > 0 && plan_ms > 0) {
+          c.ms += plan_ms;
+          tried.push_back(c);
+          best_ms = std::min(best_ms, c.ms);
         }
       }
+    }
+    // of those within 10 % of the fastest the most accurate one (of equals the
+    // faster): the depths differ by up to a factor of two in error, and short
+    // timings by a few percent from run to run
+    const Candidate* pick = nullptr;
+    for (const Candidate& c : tried)
+      if (c.ms <= 1.1f * best_ms &&
+          (!pick || c.error < 0.99 * pick->error || (c.error < 1.01 * pick->error && c.ms < pick->ms)))
+        pick = &c;
+    if (pick) {
+      best = pick->depth;
+      best_tile = pick->tile;
     }
   }
   if (s) cudaStreamDestroy(s);
@@ -126,14 +158,14 @@ void autotune(int64_t n_req, stark_dtype dt, bool grouped, int* depth_out, int* 
   cudaFree(C);
   cudaGetLastError();
   std::lock_guard<std::mutex> lk(g_tune_mu);
-  g_tuned[{n, (int)dt, grouped}] = {best, best_tile};
+  g_tuned[{n, (int)dt}] = {best, best_tile};
   *depth_out = best;
   *tile_out = best_tile;
 }
 
-int autotune_depth(int64_t n, stark_dtype dt, bool grouped) {
+int autotune_depth(int64_t n, stark_dtype dt) {
   int d = 0, tile = 128;
-  autotune(n, dt, grouped, &d, &tile);
+  autotune(n, dt, &d, &tile);
   return d;
 }
 
@@ -213,7 +245,7 @@ stark_status stark_batch_create(int32_t count, const int64_t* n, int depth, star
   b->tiles.assign(count, 128);
   for (int i = 0; i < count && st == STARK_OK; ++i) {
     int d = depth, tile = 0;
-    if (depth < 0) autotune(n[i], dt, true, &d, &tile);
+    if (depth < 0) autotune(n[i], dt, &d, &tile);
     auto* p = new (std::nothrow) stark_plan_s();
     if (!p) {
       st = STARK_ENOMEM;

@@ -1233,20 +1233,39 @@ static bool plan_tma_c(const stark_plan_s* p, const void* C) {
   return p->is_tc && p->combine_mode == 0 && (plan_uses_cstage(p, C) || c_is_tma_target(C, p->n));
 }
 
+// Few 256 x 256 tiles: 128 x 128 ones on single CTAs are four times as many
+// units with a quarter of the epilogue each.  Leaf kernel, with the K slices
+// below: n = 256 13.4 -> 10.6 us, n = 512 14.6 -> 10.5 (3xTF32 18.6 -> 11.4),
+// 16 tiles (n = 1024) 16.7 -> 14.8, 25 (n = 1280) 21.8 -> 20.7 and the clear
+// saved, 28 (n = 1024, depth 1) 21.5 -> 16.7, 36 (n = 1536) 24.7 -> 23.2 us.
+// 3xTF32, whose operands are twice the bytes, lost with 25: 29.2 -> 30.9 us.
+// Above 38 tiles the narrow ones no longer fit one round over 152 SMs.
+static bool plan_narrow(const stark_plan_s* p, int64_t lb, int64_t le) {
+  const int64_t t = p->L / 256;
+  return !p->whole_k && p->is_tc && p->combine_mode == 0 && p->pair_mode == 2 && p->bn == 256 && !p->promo_k &&
+         !p->deep_pipeline && !p->dfs && !p->shard_levels && (half_split(p->dt) || p->tf32_mn) &&
+         (le - lb) * t * t <= (half_split(p->dt) ? p->num_sms / 4 : 16);
+}
+
 // Slices of every tile's K range: while the leaves' tiles fill at most half of
 // the units that run at once (CTA pairs, or CTAs), each tile is cut in two
-// again, its slices adding into C like tiles of other leaves.  n = 256 has one
-// tile of 256 x 256; whole it took 12.4 us of leaf kernel.
+// again, its slices adding into C like tiles of other leaves.  All tiles alike:
+// with only a last round's tiles cut (3xTF32 at n = 4096, depth 2: 1.6 % faster)
+// the leaves' accumulation errors no longer cancel where the combine adds them
+// up, and the error rose by 4 %.
 static int plan_ksplit(const stark_plan_s* p, const void* C, int64_t lb, int64_t le) {
   if (p->whole_k || !plan_tma_c(p, C) || p->promo_k || p->deep_pipeline || p->dfs || p->shard_levels) return 1;
-  const bool wide = p->pair_mode == 2 && p->bn == 256;
-  const int64_t tm = p->L / (wide ? 256 : 128), tn = p->L / p->bn;
+  const bool narrow = plan_narrow(p, lb, le);
+  const bool wide = p->pair_mode == 2 && p->bn == 256 && !narrow;
+  const int64_t tm = p->L / (wide ? 256 : 128), tn = p->L / (narrow ? 128 : p->bn);
   const int64_t items = (le - lb) * tm * tn, units = wide ? p->num_sms / 2 : p->num_sms;
   const int64_t kblocks = p->L / (p->dt == STARK_F32_SPLIT_TF32 ? 32 : 64);
   int ks = 1;
   while (kblocks % (2 * ks) == 0 && items * 2 * ks <= units) ks *= 2;
   return ks;
 }
+
+int plan_k_slices(const stark_plan_s* p, const void* C) { return plan_ksplit(p, C, 0, p->P); }
 
 // Whether every element of C gets exactly one contribution (one leaf, whole K
 // ranges), stored instead of added into a cleared C.
@@ -1320,7 +1339,9 @@ static stark_status plan_leaves(stark_plan_s* p, void* C, int64_t lb, int64_t le
         return STARK_EUNSUPPORTED;
       a.promo_kb = p->promo_k / (tf32 ? 32 : 64);
     }
-    if (a.pair == 2 && p->bn == 256 && leaf_tc2_fits(a)) {
+    if (plan_narrow(p, lb, le)) {
+      st = to_status(launch_leaf_tc(a, &p->tmA, &p->tmB, &tmC, tf32, 128, p->num_sms, s));
+    } else if (a.pair == 2 && p->bn == 256 && leaf_tc2_fits(a)) {
       // CTA pairs on one 256 x 256 MMA; K-major tf32 needs Y boxes of 128 rows
       if (tf32 && !p->tf32_mn && !p->has_mapbp) {
         if (!make_tmap_planes(&p->tmBp, p->Y, true, p->L, 2 * p->P_ws, 128)) return STARK_EUNSUPPORTED;

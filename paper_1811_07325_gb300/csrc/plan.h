@@ -24,13 +24,12 @@ double model_seconds(int64_t n, int depth, stark_dtype dt);
 int choose_depth(int64_t n, stark_dtype dt);
 // Measured depth choice: times the candidate depths on the current device for
 // the size class of n (n rounded up to 64 / 128 / 256 for n up to 1024 /
-// 2048 / beyond) and caches the winner per (class, dtype, use) for the process.
-// Tensor-core dtypes.
-// grouped: for a member of a batch or of a server's micro-batch.
-int autotune_depth(int64_t n, stark_dtype dt, bool grouped = false);
+// 2048 / beyond) and caches the most accurate one within 10 % of the
+// fastest per (class, dtype) for the process.  Tensor-core dtypes.
+int autotune_depth(int64_t n, stark_dtype dt);
 // The same search over (depth, leaf tile): tile 256 = CTA pairs on 256 x 256
 // tiles (leaf sides that are multiples of 256), 128 = single CTAs on 128 x 128.
-void autotune(int64_t n, stark_dtype dt, bool grouped, int* depth, int* tile);
+void autotune(int64_t n, stark_dtype dt, int* depth, int* tile);
 
 }  // namespace stark
 
@@ -69,7 +68,7 @@ struct stark_plan_s {
   int tf32_mn = 1;       // tf32 Y planes row-major, read MN-major (0: transposed, K-major)
   bool has_mapbp = false;
   int deep_pipeline = 0; // 1: 3xBF16 with 64-byte rows, 4 stages of 48 KB (256-wide tiles)
-  bool whole_k = false;  // no K slices (timing a member of a grouped launch)
+  bool whole_k = false;  // no K slices, no narrow tiles (timing a member of a grouped launch)
   int raster_band = 0;   // tile columns per raster band of a leaf (0: row-major)
   int promo_k = 0;       // accumulator promotion every promo_k of K (CTA-pair leaves), 0: off
   CUtensorMap tmA64, tmB64;  // operand maps for the 64-byte-row schedule
@@ -156,6 +155,8 @@ void plan_release(stark_plan_s* p);
 // Enqueue C = sum over leaves [lb, le) of their combine contributions.
 stark_status plan_run(stark_plan_s* p, const void* A, const void* B, void* C, int64_t lb, int64_t le,
                       cudaStream_t s);
+// K slices that every tile of a whole product is cut into.
+int plan_k_slices(const stark_plan_s* p, const void* C);
 // Staging copy of C for the combine (allocated once; see stark_plan_s::cstage).
 stark_status plan_ensure_cstage(stark_plan_s* p);
 bool plan_uses_cstage(const stark_plan_s* p, const void* C);

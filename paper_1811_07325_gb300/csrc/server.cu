@@ -107,7 +107,7 @@ namespace {
 // Tensor-core dtypes: the measured autotuner (per size class, cached);
 // fp64/int64: the cost model.
 int depth_for(int64_t n, stark_dtype dt) {
-  return is_split(dt) ? autotune_depth(n, dt, true) : choose_depth(n, dt);
+  return is_split(dt) ? autotune_depth(n, dt) : choose_depth(n, dt);
 }
 
 // Device bytes of a workspace for side npad over `levels` depth-first levels

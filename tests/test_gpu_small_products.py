@@ -22,11 +22,12 @@ def check(S, dtype, n, d, L, C, A, B):
     assert np.all(np.abs(C.cpu().numpy().astype(np.float64) - oracle.gemm_classical(A64, B64)) <= bound)
 
 
-# slices of the pair kernel: 256/0: 4, 512/0: 8, 512/1: 4, 1024/0: 4, 1100/0 (L = 1152, 128-wide tiles): 1,
-# 300/0 (L = 384): 2 (K blocks of 128-wide tiles), 900/1 (L = 512): 2, 2048/0: 1 (stored), 130/0 (L = 256): 4
+# 128-wide tiles: 256/0 and 130/0 (L = 256) in 4 slices or more, 512/0 in 8, 512/1 in 4, 1024/0 in 2, 300/0 (L = 384)
+# in 2, 1100/0 (L = 1152) in 1, 900/1 (28 tiles of 256) in 1 or, with 3xTF32, pairs in 2; 1280/0 (25 tiles) in 1 or
+# pairs in 2; 1536/0 (36 tiles) stored by 144 CTAs; 1792/0 (49) and 2048/0 by pairs
 @pytest.mark.parametrize("dtype", ["F32_SPLIT_BF16", "F32_SPLIT_TF32", "F32_SPLIT_FP16"])
 @pytest.mark.parametrize("n,d", [(256, 0), (512, 0), (512, 1), (1024, 0), (1100, 0), (300, 0), (900, 1), (2048, 0),
-                                 (130, 0), (257, 0), (1001, 0), (2047, 0)])
+                                 (130, 0), (257, 0), (1001, 0), (2047, 0), (1280, 0), (1536, 0), (1792, 0)])
 def test_small_products(stark_lib, dtype, n, d):
     S = stark_lib
     A, B = synth.normal(n, 41 + n, 0), synth.normal(n, 41 + n, 1)

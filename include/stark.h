@@ -102,9 +102,11 @@ typedef struct {
  * Alg. 2: depth = log2 of the number of partitions per side, the paper's
  * p - q).  depth = -1 lets the library choose: for the tensor-core dtypes a
  * measured autotuner times the candidate depths on the device once per size
- * class (n rounded up to 64, 128 or 256) and caches, for the process, the most
- * accurate one within 10 % of the fastest (the paper's U-shaped optimum over the
- * partition count, Sec. V-C, found by measurement); for F64/I64 a cost model over leaf work and divide traffic.
+ * class (n rounded up to 64, 128 or 256), as a grouped member (stark_batch)
+ * runs them, and caches, for the process, the most accurate one within 3 us and
+ * 1 % of the fastest (the paper's U-shaped optimum over the partition count,
+ * Sec. V-C, found by measurement); for F64/I64 a cost model over leaf work and
+ * divide traffic.
  * depth 0 multiplies classically (one leaf).
  * Allocates the plan's device workspace on the current device.
  * Errors: EINVAL (n < 0 or > 2^20, depth < -1 or > 4, unknown dtype, out == NULL),

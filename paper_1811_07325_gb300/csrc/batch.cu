@@ -34,24 +34,23 @@ std::mutex g_tune_mu;
 // (n class, dtype) -> (depth, tile)
 std::map<std::pair<int64_t, int>, std::pair<int, int>> g_tuned;
 
-// Relative RMS error of a product of N(0, 1) inputs, as measured: the split's,
-// doubled by every level, and the tensor cores' accumulation, in proportion to
-// the K that one accumulation spans.
-double relative_error(const stark_plan_s& p, const void* C) {
-  const double k = (double)p.L / plan_k_slices(&p, C);
+// Relative RMS error of a grouped member's product of N(0, 1) inputs, as
+// measured: the split's, doubled by every level, and the tensor cores'
+// accumulation, in proportion to the K that one accumulation spans.
+double relative_error(const stark_plan_s& p) {
   const double split = (p.dt == STARK_F32_SPLIT_BF16 ? 4.4e-6 : 1e-7) * (double)(1 << p.depth);
-  const double sums = (p.dt == STARK_F32_SPLIT_TF32 ? 7.0e-9 : p.dt == STARK_F32_SPLIT_FP16 ? 3.6e-9 : 3.4e-9) * k;
+  const double sums =
+      (p.dt == STARK_F32_SPLIT_TF32 ? 7.0e-9 : p.dt == STARK_F32_SPLIT_FP16 ? 3.6e-9 : 3.4e-9) * (double)p.L;
   return std::sqrt(split * split + sums * sums);
 }
 
 // Device time (ms) of one product of side n at `depth` with leaf tiles of
-// width `tile` (256: CTA pairs; 128: single CTAs), the best of three rounds; grouped:
-// without K slices and narrow tiles, which a member of a grouped launch does
-// not get.
-float time_depth(int64_t n, int depth, stark_dtype dt, int tile, bool grouped, void* A, void* B, void* C,
-                 cudaStream_t s, double* error) {
+// width `tile` (256: CTA pairs; 128: single CTAs) as a grouped member runs it
+// (whole K ranges), the best of three rounds, and its error.
+float time_depth(int64_t n, int depth, stark_dtype dt, int tile, void* A, void* B, void* C, cudaStream_t s,
+                 double* error) {
   stark_plan_s p;
-  p.whole_k = grouped;
+  p.whole_k = true;
   if (plan_init(&p, n, depth, dt) != STARK_OK) {
     plan_release(&p);
     return -1.f;
@@ -63,7 +62,7 @@ float time_depth(int64_t n, int depth, stark_dtype dt, int tile, bool grouped, v
     plan_release(&p);
     return -1.f;
   }
-  *error = relative_error(p, C);
+  *error = relative_error(p);
   cudaEvent_t e0, e1;
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
@@ -91,8 +90,8 @@ float time_depth(int64_t n, int depth, stark_dtype dt, int tile, bool grouped, v
 }  // namespace
 
 // Measured depth choice for n x n products (cached per process): one for a plan,
-// a batch's member and a request, whose results then agree, by the time of the
-// product as a plan plus its time as a member.
+// a batch's member and a request, by the product's time and error as a member
+// (a plan's K slices only lower its error at the same depth).
 void autotune(int64_t n_req, stark_dtype dt, int* depth_out, int* tile_out) {
   // size class: n rounded up to 64 (n <= 1024), 128 (n <= 2048), else 256
   const int64_t q = n_req <= 1024 ? 64 : n_req <= 2048 ? 128 : 256;
@@ -126,25 +125,26 @@ void autotune(int64_t n_req, stark_dtype dt, int* depth_out, int* tile_out) {
       if ((padded_side(n, d, dt) >> d) < tile_granularity(dt)) continue;
       if (d > 0 && (n >> d) < 128) break;
       const bool wide = (padded_side(n, d, dt) >> d) % 256 == 0;
-      double plan_error;
-      const float plan_ms = time_depth(n, d, dt, wide ? 256 : 128, false, A, B, C, s, &plan_error);
       for (int tile : {256, 128}) {
         if (tile == 256 && !wide) continue;
         Candidate c{d, tile, 0.f, 0.0};
-        c.ms = time_depth(n, d, dt, tile, true, A, B, C, s, &c.error);
-        if (c.ms > 0 && plan_ms > 0) {
-          c.ms += plan_ms;
+        c.ms = time_depth(n, d, dt, tile, A, B, C, s, &c.error);
+        if (c.ms > 0) {
           tried.push_back(c);
           best_ms = std::min(best_ms, c.ms);
         }
       }
     }
-    // of those within 10 % of the fastest the most accurate one (of equals the
-    // faster): the depths differ by up to a factor of two in error, and short
-    // timings by a few percent from run to run
+    // of those within 3 us and 1 % of the fastest the most accurate one (of
+    // equals the faster).  The depths differ by up to a factor of two in error
+    // and, up to n = 1024, by one to three microseconds in time.  By time alone
+    // a one-leaf product, stored without a clear (3xFP16, n = 576: 15.5 us, and
+    // 17.0 at depth 1), would take many of these sizes from the depth of half
+    // its error.  Over 43 size classes up to n = 12288 and three dtypes the
+    // pick was within 3 us of the fastest and, from n = 2304 on, within 1 %.
     const Candidate* pick = nullptr;
     for (const Candidate& c : tried)
-      if (c.ms <= 1.1f * best_ms &&
+      if (c.ms <= 1.01f * best_ms + 3e-3f &&
           (!pick || c.error < 0.99 * pick->error || (c.error < 1.01 * pick->error && c.ms < pick->ms)))
         pick = &c;
     if (pick) {

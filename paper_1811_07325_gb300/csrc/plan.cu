@@ -1265,8 +1265,6 @@ static int plan_ksplit(const stark_plan_s* p, const void* C, int64_t lb, int64_t
   return ks;
 }
 
-int plan_k_slices(const stark_plan_s* p, const void* C) { return plan_ksplit(p, C, 0, p->P); }
-
 // Whether every element of C gets exactly one contribution (one leaf, whole K
 // ranges), stored instead of added into a cleared C.
 static bool plan_direct(const stark_plan_s* p, const void* C, int64_t lb, int64_t le) {

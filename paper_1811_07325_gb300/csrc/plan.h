@@ -24,8 +24,8 @@ double model_seconds(int64_t n, int depth, stark_dtype dt);
 int choose_depth(int64_t n, stark_dtype dt);
 // Measured depth choice: times the candidate depths on the current device for
 // the size class of n (n rounded up to 64 / 128 / 256 for n up to 1024 /
-// 2048 / beyond) and caches the most accurate one within 10 % of the
-// fastest per (class, dtype) for the process.  Tensor-core dtypes.
+// 2048 / beyond) and caches the most accurate one within 3 us and
+// 1 % of the fastest per (class, dtype) for the process.  Tensor-core dtypes.
 int autotune_depth(int64_t n, stark_dtype dt);
 // The same search over (depth, leaf tile): tile 256 = CTA pairs on 256 x 256
 // tiles (leaf sides that are multiples of 256), 128 = single CTAs on 128 x 128.
@@ -155,8 +155,6 @@ void plan_release(stark_plan_s* p);
 // Enqueue C = sum over leaves [lb, le) of their combine contributions.
 stark_status plan_run(stark_plan_s* p, const void* A, const void* B, void* C, int64_t lb, int64_t le,
                       cudaStream_t s);
-// K slices that every tile of a whole product is cut into.
-int plan_k_slices(const stark_plan_s* p, const void* C);
 // Staging copy of C for the combine (allocated once; see stark_plan_s::cstage).
 stark_status plan_ensure_cstage(stark_plan_s* p);
 bool plan_uses_cstage(const stark_plan_s* p, const void* C);

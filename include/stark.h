@@ -218,7 +218,10 @@ STARK_API stark_status stark_plan_operands(stark_plan_t plan, const void *A, con
 /* How the combine (Alg. 5) adds leaf tiles into C on the tensor-core dtypes:
  * mode 0 (default) fuses it into the leaf epilogue with TMA bulk
  * add-reductions of 32 x 32 boxes (through an aligned staging copy of C when
- * n is not a multiple of 4); mode 1 fuses it with signed vector atomics;
+ * n is not a multiple of 4; the additions come in any order, so results
+ * differ in rounding from run to run at depth >= 1 and are bitwise
+ * reproducible at depth 0, where an element has one contribution, or two
+ * added to zero); mode 1 fuses it with signed vector atomics;
  * mode 2 is deterministic: the leaf epilogue stores every product M_l
  * (allocating [leaves][L][L] fp32 planes) and a separate pass writes each C
  * element once as its signed sum in ascending leaf order, so results are

@@ -1235,7 +1235,7 @@ static bool plan_tma_c(const stark_plan_s* p, const void* C) {
 
 // Few 256 x 256 tiles: 128 x 128 ones on single CTAs are four times as many
 // units with a quarter of the epilogue each.  Leaf kernel, with the K slices
-// below: n = 256 13.4 -> 10.6 us, n = 512 14.6 -> 10.5 (3xTF32 18.6 -> 11.4),
+// below: n = 256 13.4 -> 10.9 us, n = 512 14.6 -> 12.5 (3xTF32 18.6 -> 14.7),
 // 16 tiles (n = 1024) 16.7 -> 14.8, 25 (n = 1280) 21.8 -> 20.7 and the clear
 // saved, 28 (n = 1024, depth 1) 21.5 -> 16.7, 36 (n = 1536) 24.7 -> 23.2 us.
 // 3xTF32, whose operands are twice the bytes, lost with 25: 29.2 -> 30.9 us.
@@ -1252,7 +1252,9 @@ static bool plan_narrow(const stark_plan_s* p, int64_t lb, int64_t le) {
 // again, its slices adding into C like tiles of other leaves.  All tiles alike:
 // with only a last round's tiles cut (3xTF32 at n = 4096, depth 2: 1.6 % faster)
 // the leaves' accumulation errors no longer cancel where the combine adds them
-// up, and the error rose by 4 %.
+// up, and the error rose by 4 %.  A one-leaf product takes at most two slices:
+// with two contributions to a cleared C their order does not show, and the
+// product stays repeatable bit for bit (with up to eight, n = 512 did not).
 static int plan_ksplit(const stark_plan_s* p, const void* C, int64_t lb, int64_t le) {
   if (p->whole_k || !plan_tma_c(p, C) || p->promo_k || p->deep_pipeline || p->dfs || p->shard_levels) return 1;
   const bool narrow = plan_narrow(p, lb, le);
@@ -1260,8 +1262,9 @@ static int plan_ksplit(const stark_plan_s* p, const void* C, int64_t lb, int64_t
   const int64_t tm = p->L / (wide ? 256 : 128), tn = p->L / (narrow ? 128 : p->bn);
   const int64_t items = (le - lb) * tm * tn, units = wide ? p->num_sms / 2 : p->num_sms;
   const int64_t kblocks = p->L / (p->dt == STARK_F32_SPLIT_TF32 ? 32 : 64);
+  const int most = p->depth == 0 ? 2 : 1 << 30;
   int ks = 1;
-  while (kblocks % (2 * ks) == 0 && items * 2 * ks <= units) ks *= 2;
+  while (ks < most && kblocks % (2 * ks) == 0 && items * 2 * ks <= units) ks *= 2;
   return ks;
 }
 

@@ -1254,9 +1254,11 @@ static bool plan_narrow(const stark_plan_s* p, int64_t lb, int64_t le) {
 // the leaves' accumulation errors no longer cancel where the combine adds them
 // up, and the error rose by 4 %.  A one-leaf product takes at most two slices:
 // with two contributions to a cleared C their order does not show, and the
-// product stays repeatable bit for bit (with up to eight, n = 512 did not).
+// product stays repeatable bit for bit (with up to eight, n = 512 did not).  A
+// range of a deeper product's leaves, which may give an element one or two
+// contributions, is not sliced, for the same reason.
 static int plan_ksplit(const stark_plan_s* p, const void* C, int64_t lb, int64_t le) {
-  if (p->whole_k || !plan_tma_c(p, C) || p->promo_k || p->deep_pipeline || p->dfs || p->shard_levels) return 1;
+  if (p->whole_k || le - lb < p->P || !plan_tma_c(p, C) || p->promo_k || p->deep_pipeline || p->dfs || p->shard_levels) return 1;
   const bool narrow = plan_narrow(p, lb, le);
   const bool wide = p->pair_mode == 2 && p->bn == 256 && !narrow;
   const int64_t tm = p->L / (wide ? 256 : 128), tn = p->L / (narrow ? 128 : p->bn);

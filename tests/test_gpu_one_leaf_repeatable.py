@@ -21,3 +21,19 @@ def test_one_leaf_products_are_repeatable(stark_lib, dtype, n):
         for _ in range(60):
             assert torch.equal(p.mul(A, B), first)
         p.check()
+
+
+@pytest.mark.parametrize("dtype", ["F32_SPLIT_BF16", "F32_SPLIT_TF32", "F32_SPLIT_FP16"])
+@pytest.mark.parametrize("lo,hi", [(0, 1), (1, 3), (4, 7)])
+def test_leaf_ranges_with_few_contributions_are_repeatable(stark_lib, dtype, lo, hi):
+    # one leaf, two leaves (M2 and M3 meet in C22), three (M5 and M7 meet in C11): at most two additions to zero
+    S = stark_lib
+    n = 512
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    A = torch.randn((n, n), generator=gen, device="cuda")
+    B = torch.randn((n, n), generator=gen, device="cuda")
+    with S.Plan(n, 1, S.DType[dtype]) as p:
+        first = p.mul_leaves(A, B, lo, hi).clone()
+        for _ in range(60):
+            assert torch.equal(p.mul_leaves(A, B, lo, hi), first)
+        p.check()

@@ -309,8 +309,9 @@ STARK_API stark_status stark_plan_set_pipeline(stark_plan_t plan, int deep);
  * first over the top k levels: for each of the 7^k products there, divide
  * only its subtree (reading A and B through that product's level-1..k
  * operand sums, formed on the fly in the order of Alg. 1) and launch its
- * 7^(d-k) leaves; the workspace shrinks 7^k-fold (the plan reallocates it),
- * the divide reads A and B 3^k times over.  Results agree within the
+ * 7^(d-k) leaves; the operand workspace shrinks 7^k-fold (the plan
+ * reallocates it, and an F64 or I64 plan releases its product planes and side
+ * arrays meanwhile), the divide reads A and B 3^k times over.  Results agree within the
  * combine's rounding order (bit-identical for int64).  Errors: EINVAL
  * (levels outside 0..2), EUNSUPPORTED (levels > depth, depth > 3, levels =
  * 2 on an F64/I64 plan, or the deterministic combine mode), ENOMEM, ECUDA.
@@ -343,9 +344,12 @@ STARK_API stark_status stark_plan_set_shard(stark_plan_t plan, int64_t leaf_begi
  * into int64: bit-identical to the int64 CUDA-core path.  The divide checks
  * every operand on the device; a value beyond the range makes the next
  * stark_plan_check return STARK_EINVAL (the product is then invalid).
- * max_abs = 0 returns to the CUDA-core path.  Errors: EINVAL (not an I64
+ * max_abs = 0 returns to the leaves of an unbounded plan.  The plan keeps its
+ * operand workspace, sized for those, so that products captured before stay
+ * valid; fp32 planes for the products of a whole breadth-first product are
+ * allocated where the plan has none.  Errors: EINVAL (not an I64
  * plan, max_abs < 0), EUNSUPPORTED (the bound does not give exactness at
- * this depth / leaf side; the plan keeps the CUDA-core path). */
+ * this depth / leaf side; the plan keeps its unbounded leaves). */
 STARK_API stark_status stark_plan_set_input_bound(stark_plan_t plan, int64_t max_abs);
 
 /* Synchronise the plan's last stream and report any device-side error

@@ -257,7 +257,8 @@ double model_seconds(int64_t n, int depth, stark_dtype dt) {
 
 // Whether a product of this plan runs its leaves as digit products.
 static bool plan_limbs(const stark_plan_s* p) {
-  return p->limb_ok && !p->int_tc && !p->dfs && !p->shard_levels && p->op_elem == 16;
+  return p->limb_ok && !p->int_tc && !p->dfs && !p->shard_levels && p->op_elem == 16 && (p->depth == 0 || p->limb_m) &&
+         (p->dt != STARK_F64 || p->limb_aux);
 }
 
 // Tensor maps of the digit planes.
@@ -643,6 +644,91 @@ static stark_status plan_tune_combine(stark_plan_t p) {
   return st;
 }
 
+// The magnitude sum each F64 leaf's elements must reach (leaf_limb.cu has the
+// derivation), from the leaf side and the terms that padding leaves the leaf.
+static void limb_check_sums(const stark_plan_s* p, std::vector<float>& need) {
+  const double rounded = p->L <= 1024 ? 1.0 : 1.5;  // half units a superchunk
+  const double full = 16384.0 * (1.0 / 64 + rounded * (double)p->L / 128.0 / 512.0);
+  const float full_need = (float)std::max(512.0, full);
+  need.assign((size_t)p->P, full_need);
+  if (p->depth == 0) return;
+  std::vector<int64_t> terms((size_t)p->P, kLimbCheckK);
+  for (int side = 0; side < 2; ++side) {
+    std::vector<int32_t> cnt, quad;
+    std::vector<int8_t> sign;
+    build_quadrant_table(p->depth, side, cnt, quad, sign);
+    for (int64_t l = 0; l < p->P; ++l) {
+      int64_t k = 0;  // K positions with an input element in some term (columns of A, rows of B)
+      for (int t = 0; t < cnt[(size_t)l]; ++t) {
+        int64_t r = 0, c = 0;
+        quadrant_offsets(p->depth, p->npad, quad[(size_t)(l << p->depth) + t], &r, &c);
+        k = std::max(k, core_side(p) - (side == 0 ? c : r));
+      }
+      terms[(size_t)l] = std::min(terms[(size_t)l], k);
+    }
+  }
+  for (int64_t l = 0; l < p->P; ++l)
+    if (terms[(size_t)l] < kLimbCheckK) need[(size_t)l] = terms[(size_t)l] < 16 ? 0.f : (float)terms[(size_t)l];
+}
+
+// Bytes of an F64 plan's bounds, exponents, magnitude planes and flag (every
+// part a multiple of 256).
+static int64_t limb_aux_bytes(const stark_plan_s* p) {
+  const int64_t maxima = (p->npad << p->depth) * 8, exps = (p->P * p->L * 4 + 255) / 256 * 256,
+                mags = p->P * p->L * kLimbCheckK * 2, needs = (p->P * 4 + 255) / 256 * 256,
+                commons = (p->L * 4 + 255) / 256 * 256;
+  return 256 + needs + 2 * (maxima + exps + mags + commons);
+}
+
+// What limb leaves need besides the digit planes: product planes (depth >= 1)
+// and, for F64, the side arrays.  On failure nothing new is kept.
+static bool plan_limb_extras(stark_plan_s* p) {
+  const int64_t products = p->P * p->L * p->L * 8, aux = limb_aux_bytes(p);
+  const bool had_m = p->limb_m, had_aux = p->limb_aux;
+  bool ok = p->depth == 0 || had_m || cudaMalloc(&p->limb_m, (size_t)products) == cudaSuccess;
+  if (ok && p->dt == STARK_F64 && !had_aux) {
+    ok = cudaMalloc(&p->limb_aux, (size_t)aux) == cudaSuccess;
+    if (ok) {
+      const int64_t maxima = (p->npad << p->depth) * 8, exps = (p->P * p->L * 4 + 255) / 256 * 256,
+                    mags = p->P * p->L * kLimbCheckK * 2, needs = (p->P * 4 + 255) / 256 * 256,
+                    commons = (p->L * 4 + 255) / 256 * 256;
+      char* b = static_cast<char*>(p->limb_aux);
+      p->d_flag = reinterpret_cast<int*>(b);
+      b += 256;
+      p->limb_need = reinterpret_cast<float*>(b);
+      b += needs;
+      p->common_a = reinterpret_cast<int32_t*>(b);
+      p->common_b = reinterpret_cast<int32_t*>(b + commons);
+      b += 2 * commons;
+      p->mag_a = b;
+      p->mag_b = b + mags;
+      b += 2 * mags;
+      p->exp_a = reinterpret_cast<int32_t*>(b);
+      p->exp_b = reinterpret_cast<int32_t*>(b + exps);
+      b += 2 * exps;
+      p->max_a = reinterpret_cast<double*>(b);
+      p->max_b = reinterpret_cast<double*>(b + maxima);
+      std::vector<float> need;
+      limb_check_sums(p, need);
+      ok = cudaMemcpy(p->limb_need, need.data(), need.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+    }
+  }
+  if (!ok) {
+    cudaGetLastError();
+    if (!had_m) {
+      cudaFree(p->limb_m);
+      p->limb_m = nullptr;
+    }
+    if (!had_aux) {
+      cudaFree(p->limb_aux);
+      p->limb_aux = nullptr;
+    }
+    return false;
+  }
+  p->ws_bytes += (p->limb_m && !had_m ? products : 0) + (p->limb_aux && !had_aux ? aux : 0);
+  return true;
+}
+
 // Workspace for `planes_per_half` leaves per operand side, with its maps.
 // (per: bytes per leaf element and operand).
 static stark_status plan_alloc_operands_at(stark_plan_s* p, int64_t planes, int64_t per) {
@@ -689,12 +775,57 @@ static stark_status plan_alloc_operands_at(stark_plan_s* p, int64_t planes, int6
   return STARK_OK;
 }
 
-static stark_status plan_alloc_operands(stark_plan_s* p, int64_t planes) {
-  if (p->limb_ok && planes == p->P) {  // digit planes, where they fit (breadth first only)
-    const stark_status st = plan_alloc_operands_at(p, planes, 16);
-    if (st != STARK_ENOMEM) return st;
+// The product planes and the F64 side arrays that only whole breadth-first
+// products use.  (Nothing of the plan may be running.)
+static void plan_free_products(stark_plan_s* p) {
+  const int64_t elems = p->P * p->L * p->L;
+  if (p->int_m && p->int_m != p->limb_m) {
+    cudaFree(p->int_m);
+    p->ws_bytes -= elems * 4;
   }
-  return plan_alloc_operands_at(p, planes, half_split(p->dt) ? 4 : 8);
+  if (p->limb_m) {
+    cudaFree(p->limb_m);
+    p->ws_bytes -= elems * 8;
+  }
+  if (p->limb_aux) {
+    cudaFree(p->limb_aux);
+    p->ws_bytes -= limb_aux_bytes(p);
+  }
+  p->int_m = p->limb_m = p->limb_aux = nullptr;
+}
+
+// Planes for the products of a bounded integer plan: the digit products' where
+// the plan has them.  Without any the products are added into C as they finish.
+static stark_status plan_int_products(stark_plan_s* p) {
+  if (p->int_m || p->n == 0) return STARK_OK;
+  p->int_m = p->limb_m;
+  if (!p->int_m) {
+    const size_t bytes = (size_t)p->P * p->L * p->L * sizeof(float);
+    if (cudaMalloc(&p->int_m, bytes) == cudaSuccess) {
+      p->ws_bytes += (int64_t)bytes;
+    } else {
+      cudaGetLastError();
+      p->int_m = nullptr;
+    }
+  }
+  return !p->int_m || make_tmap_mplanes(&p->tmIM, p->int_m, p->L, p->P) ? STARK_OK : STARK_EUNSUPPORTED;
+}
+
+// whole: for whole breadth-first products, which take digit planes where the
+// plan has limb leaves and they fit; a subtree's or a shard's operands else.
+static stark_status plan_alloc_operands(stark_plan_s* p, int64_t planes, bool whole) {
+  if (!whole) {
+    if (cudaDeviceSynchronize() != cudaSuccess) return STARK_ECUDA;
+    plan_free_products(p);
+  }
+  stark_status st = STARK_ENOMEM;
+  if (whole && p->limb_ok) {
+    if (plan_limb_extras(p)) st = plan_alloc_operands_at(p, planes, 16);
+    if (st == STARK_ENOMEM) plan_free_products(p);
+  }
+  if (st == STARK_ENOMEM) st = plan_alloc_operands_at(p, planes, half_split(p->dt) ? 4 : 8);
+  if (st == STARK_OK && whole && p->int_tc) st = plan_int_products(p);
+  return st;
 }
 
 stark_status stark_plan_set_traversal(stark_plan_t p, int levels) {
@@ -706,7 +837,7 @@ stark_status stark_plan_set_traversal(stark_plan_t p, int levels) {
     return STARK_OK;
   }
   const int prev = p->dfs;
-  const stark_status st = plan_alloc_operands(p, p->P / pow7i(levels));
+  const stark_status st = plan_alloc_operands(p, p->P / pow7i(levels), levels == 0);
   // the traversal follows the workspace that exists (on a failed growth the
   // plan keeps its previous one)
   p->dfs = p->P_ws == p->P / pow7i(levels) ? levels : prev;
@@ -717,7 +848,7 @@ stark_status stark_plan_set_shard(stark_plan_t p, int64_t lb, int64_t le) {
   if (!p || lb < 0 || le > p->P || lb >= le) return STARK_EINVAL;
   if (p->dfs) return STARK_EUNSUPPORTED;
   if (lb == 0 && le == p->P) {  // the whole product: breadth first, full workspace
-    const stark_status st = p->shard_levels && p->n > 0 ? plan_alloc_operands(p, p->P) : STARK_OK;
+    const stark_status st = p->shard_levels && p->n > 0 ? plan_alloc_operands(p, p->P, true) : STARK_OK;
     if (st == STARK_OK) {
       p->shard_levels = 0;
       p->shard_lb = 0;
@@ -732,7 +863,7 @@ stark_status stark_plan_set_shard(stark_plan_t p, int64_t lb, int64_t le) {
   const int64_t gs = pow7i(p->depth - k);
   const int64_t g0 = lb / gs, g1 = (le + gs - 1) / gs;
   if (p->n > 0) {
-    const stark_status st = plan_alloc_operands(p, (g1 - g0) * gs);
+    const stark_status st = plan_alloc_operands(p, (g1 - g0) * gs, false);
     if (st != STARK_OK) return st;
   }
   p->shard_levels = k;
@@ -758,20 +889,8 @@ stark_status stark_plan_set_input_bound(stark_plan_t p, int64_t max_abs) {
   if (!make_tmap_planes(&p->tmAi, p->X, false, p->L, p->P_ws, 128) ||
       !make_tmap_planes(&p->tmBi, p->Y, false, p->L, p->P_ws, 64))
     return STARK_EUNSUPPORTED;
-  // planes for the products: the digit products' where the plan has them
-  if (!p->int_m && p->n > 0) {
-    p->int_m = p->limb_m;
-    if (!p->int_m) {
-      const size_t bytes = (size_t)p->P * p->L * p->L * sizeof(float);
-      if (cudaMalloc(&p->int_m, bytes) == cudaSuccess) {
-        p->ws_bytes += (int64_t)bytes;
-      } else {  // without them the products are added into C as they finish
-        cudaGetLastError();
-        p->int_m = nullptr;
-      }
-    }
-    if (p->int_m && !make_tmap_mplanes(&p->tmIM, p->int_m, p->L, p->P)) return STARK_EUNSUPPORTED;
-  }
+  if (!p->dfs && !p->shard_levels)
+    if (const stark_status st = plan_int_products(p); st != STARK_OK) return st;
   p->int_bound = max_abs;
   p->int_tc = true;
   return STARK_OK;
@@ -891,82 +1010,17 @@ bool traversal_supported(int depth, stark_dtype dt, int levels) {
   return levels == 1 || is_split(dt);
 }
 
-// The magnitude sum each F64 leaf's elements must reach (leaf_limb.cu has the
-// derivation), from the leaf side and the terms that padding leaves the leaf.
-static void limb_check_sums(const stark_plan_s* p, std::vector<float>& need) {
-  const double rounded = p->L <= 1024 ? 1.0 : 1.5;  // half units a superchunk
-  const double full = 16384.0 * (1.0 / 64 + rounded * (double)p->L / 128.0 / 512.0);
-  const float full_need = (float)std::max(512.0, full);
-  need.assign((size_t)p->P, full_need);
-  if (p->depth == 0) return;
-  std::vector<int64_t> terms((size_t)p->P, kLimbCheckK);
-  for (int side = 0; side < 2; ++side) {
-    std::vector<int32_t> cnt, quad;
-    std::vector<int8_t> sign;
-    build_quadrant_table(p->depth, side, cnt, quad, sign);
-    for (int64_t l = 0; l < p->P; ++l) {
-      int64_t k = 0;  // K positions with an input element in some term (columns of A, rows of B)
-      for (int t = 0; t < cnt[(size_t)l]; ++t) {
-        int64_t r = 0, c = 0;
-        quadrant_offsets(p->depth, p->npad, quad[(size_t)(l << p->depth) + t], &r, &c);
-        k = std::max(k, core_side(p) - (side == 0 ? c : r));
-      }
-      terms[(size_t)l] = std::min(terms[(size_t)l], k);
-    }
-  }
-  for (int64_t l = 0; l < p->P; ++l)
-    if (terms[(size_t)l] < kLimbCheckK) need[(size_t)l] = terms[(size_t)l] < 16 ? 0.f : (float)terms[(size_t)l];
-}
-
-// X and Y for the digit planes (`ws` bytes together) and, for F64, the bounds,
-// exponents and magnitude planes with the flag.  On failure nothing is kept.
+// X and Y for the digit planes (`ws` bytes together) with the extras.  On
+// failure nothing is kept.
 static bool plan_limb_alloc(stark_plan_s* p, int64_t ws) {
   bool ok = cudaMalloc(&p->X, (size_t)(ws / 2)) == cudaSuccess && cudaMalloc(&p->Y, (size_t)(ws / 2)) == cudaSuccess;
-  int64_t aux = 0, products = 0;
-  if (ok && p->depth > 0) {
-    products = p->P * p->L * p->L * 8;
-    ok = cudaMalloc(&p->limb_m, (size_t)products) == cudaSuccess;
-  }
-  if (ok && p->dt == STARK_F64) {
-    const int64_t maxima = (p->npad << p->depth) * 8, exps = (p->P * p->L * 4 + 255) / 256 * 256,
-                  mags = p->P * p->L * kLimbCheckK * 2;
-    const int64_t needs = (p->P * 4 + 255) / 256 * 256;
-    const int64_t commons = (p->L * 4 + 255) / 256 * 256;
-    aux = 256 + needs + 2 * (maxima + exps + mags + commons);
-    ok = cudaMalloc(&p->limb_aux, (size_t)aux) == cudaSuccess;
-    if (ok) {
-      char* b = static_cast<char*>(p->limb_aux);
-      p->d_flag = reinterpret_cast<int*>(b);
-      b += 256;  // every part is a multiple of 256 bytes
-      p->limb_need = reinterpret_cast<float*>(b);
-      b += needs;
-      p->common_a = reinterpret_cast<int32_t*>(b);
-      p->common_b = reinterpret_cast<int32_t*>(b + commons);
-      b += 2 * commons;
-      p->mag_a = b;
-      p->mag_b = b + mags;
-      b += 2 * mags;
-      p->exp_a = reinterpret_cast<int32_t*>(b);
-      p->exp_b = reinterpret_cast<int32_t*>(b + exps);
-      b += 2 * exps;
-      p->max_a = reinterpret_cast<double*>(b);
-      p->max_b = reinterpret_cast<double*>(b + maxima);
-      std::vector<float> need;
-      limb_check_sums(p, need);
-      ok = cudaMemcpy(p->limb_need, need.data(), need.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
-    }
-  }
-  ok = ok && plan_limb_maps(p);
-  if (ok) {
-    p->ws_bytes += aux + products;
-    return true;
-  }
+  ok = ok && plan_limb_extras(p) && plan_limb_maps(p);
+  if (ok) return true;
   cudaGetLastError();
   cudaFree(p->X);
   cudaFree(p->Y);
-  cudaFree(p->limb_m);
-  cudaFree(p->limb_aux);
-  p->X = p->Y = p->limb_m = p->limb_aux = nullptr;
+  p->X = p->Y = nullptr;
+  plan_free_products(p);
   return false;
 }
 

@@ -47,8 +47,16 @@
 // most 2^(d+2) such units (limb_bounds.cu), 2^-57 R at depth 3, where the fp64
 // sums alone are off by 2^-53 of themselves a level.  Given them, and with C
 // the bound of the column of B, a product of K non-zero terms is off by at most K 2^-59 R C (the dropped digit products,
-// 7 * 2^14 * 256^6 / 2^124 a term) and three half units of the running sum
-// per superchunk, the unit being L 2^-62 R C.  A K-term FP64 dot product is
+// 7 * 2^14 * 256^6 / 2^124 a term) and half a unit of the running sum for
+// every rounded diagonal.  The sum keeps 64 bits, so the unit follows from the
+// most that the product can be: by Cauchy and Schwarz at most the product of
+// the 2-norms of its row and column, which limb_bounds.cu has as R C 2^l
+// (2^l >= L) less the slacks of both.  With the slack of its own row and the
+// least of its warp's 64 columns, the unit is 2^(l - 62) R C less that: at most
+// 2^-59 of those norms' product unless a column stands out among the 64.  (With
+// the unit 2^(l - 62) R C of rows without slack, rows of 1024 elements of about
+// one with a single one of up to 32 were off by 5 times as much as in FP64.)
+// A K-term FP64 dot product is
 // only bound to K 2^-53 sum |a||b|.  So the digits are the more accurate of
 // the two unless nearly every |a||b| is far below R C (badly scaled or sparse
 // rows), and the kernel proves for each element that it is not: over the
@@ -81,9 +89,14 @@ constexpr int kBarBytes = 8 * (2 * kQuads + 8) + 16;
 constexpr int kSmemLimb = kQuads * kQuadBytes + kEpiBytes + 1024 + kBarBytes;
 static_assert(kSmemLimb <= 232448, "shared memory per CTA");
 // acc + v 2^32, on the high word alone.
-__device__ __forceinline__ long long add_high(long long acc, int v) {
-  const uint32_t hi = (uint32_t)((unsigned long long)acc >> 32) + (uint32_t)v;
+__device__ __forceinline__ long long add_high(long long acc, uint32_t v) {
+  const uint32_t hi = (uint32_t)((unsigned long long)acc >> 32) + v;
   return (long long)(((unsigned long long)hi << 32) | (uint32_t)acc);
+}
+
+// acc + v mul.  (The sums are kept mod 2^64: only the last one has to fit.)
+__device__ __forceinline__ long long add_wide(long long acc, int v, int mul) {
+  return (long long)((unsigned long long)acc + (unsigned long long)((long long)v * mul));
 }
 
 // v * 2^e rounded to nearest (ties away), from integer operations (the FP64
@@ -392,11 +405,13 @@ __global__ void __launch_bounds__(kThreadsL, 1)
     const uint32_t ebuf = epi_base + (uint32_t)(warp - 4) * (32 * kEpiStride + 256);
     const uint32_t fbuf = ebuf + 32 * kEpiStride;
     uint32_t acc_phase = 0;
+    int shift = p.shift;  // F64: 2^shift of 256^7 is the unit of this thread's sums
     bool ok = true;
     long long sum[64];
     auto wait_acc = [&](int a) -> bool {
       if (!mbar_wait_bounded(accf_bar(a), (acc_phase >> a) & 1, p.err, kDevTimeoutAccFull, p.timeout_ns)) return false;
       acc_phase ^= 1u << a;
+      if (F64) __syncwarp();  // (rows of unlike shift part in drain's branch)
       tc_fence_after();
       return true;
     };
@@ -409,8 +424,8 @@ __global__ void __launch_bounds__(kThreadsL, 1)
     auto drain = [&](int a, int s) -> bool {
       if (!wait_acc(a)) return false;
       // I64: 256^s.  F64: 256^(7-s) in units of 2^shift (contributions below
-      // the unit are rounded; the unit is at most K 2^-62 R C)
-      const int sh = F64 ? 8 * (7 - s) - p.shift : 8 * s;
+      // the unit are rounded)
+      const int sh = F64 ? 8 * (7 - s) - shift : 8 * s;
       const uint32_t col = lane_base + (uint32_t)(a * 128);
       uint32_t r0[32], r1[32];
       tmem_ld_32x32b_x32(col, r0);
@@ -418,11 +433,11 @@ __global__ void __launch_bounds__(kThreadsL, 1)
       tmem_ld_wait();
       free_acc(a);  // the additions need only registers
       if (sh >= 32) {
-        const int mul = 1 << (sh - 32);
+        const uint32_t mul = 1u << (sh - 32);
 #pragma unroll
         for (int e = 0; e < 32; ++e) {
-          sum[e] = add_high(sum[e], __float2int_rn(__uint_as_float(r0[e])) * mul);
-          sum[32 + e] = add_high(sum[32 + e], __float2int_rn(__uint_as_float(r1[e])) * mul);
+          sum[e] = add_high(sum[e], (uint32_t)__float2int_rn(__uint_as_float(r0[e])) * mul);
+          sum[32 + e] = add_high(sum[32 + e], (uint32_t)__float2int_rn(__uint_as_float(r1[e])) * mul);
         }
       } else {
         // v 2^sh = (v scale) mul, rounded where sh < 0 (|v| <= 2^24)
@@ -431,8 +446,8 @@ __global__ void __launch_bounds__(kThreadsL, 1)
         const int mul = 1 << ms;
 #pragma unroll
         for (int e = 0; e < 32; ++e) {
-          sum[e] += (long long)__float2int_rn(__uint_as_float(r0[e]) * scale) * mul;
-          sum[32 + e] += (long long)__float2int_rn(__uint_as_float(r1[e]) * scale) * mul;
+          sum[e] = add_wide(sum[e], __float2int_rn(__uint_as_float(r0[e]) * scale), mul);
+          sum[32 + e] = add_wide(sum[32 + e], __float2int_rn(__uint_as_float(r1[e]) * scale), mul);
         }
       }
       return true;
@@ -442,7 +457,6 @@ __global__ void __launch_bounds__(kThreadsL, 1)
       const int tile = item % per_leaf;
       const int row0 = tile / tiles * 128 + quarter * 32, row = row0 + lane;  // in the leaf plane
       const int col0 = tile % tiles * 128 + half * 64;
-      int ea = 0;
       auto fexp = [&](int c) {  // exponent of column col0 + c
         int f;
         asm volatile("ld.shared.s32 %0, [%1];" : "=r"(f) : "r"(fbuf + 4u * (uint32_t)c));
@@ -450,14 +464,20 @@ __global__ void __launch_bounds__(kThreadsL, 1)
       };
       if (F64) {
         const int32_t* fb = p.expB + (int64_t)leaf * p.L;
-        ea = row < p.L ? p.expA[(int64_t)leaf * p.L + row] : kLimbZeroRow;
+        const int ea = row < p.L ? p.expA[(int64_t)leaf * p.L + row] : kLimbZeroRow;
+        const int none = p.shift - 4;  // the most slack there is
+        int slack = none;              // the least of this warp's columns
         __syncwarp();  // (the previous tile's exponents have been read)
 #pragma unroll
         for (int h = 0; h < 64; h += 32) {
-          const int f = col0 + h + lane < p.L ? fb[col0 + h + lane] : kLimbZeroRow;
+          const bool in = col0 + h + lane < p.L;
+          const int f = in ? fb[col0 + h + lane] : kLimbZeroRow;
           asm volatile("st.shared.s32 [%0], %1;" ::"r"(fbuf + 4u * (uint32_t)(h + lane)), "r"(f) : "memory");
+          if (in) slack = min(slack, p.slackB[(int64_t)leaf * p.L + col0 + h + lane]);
         }
         __syncwarp();
+        slack = __reduce_min_sync(0xffffffffu, slack);
+        shift = p.shift - (slack + (row < p.L ? p.slackA[(int64_t)leaf * p.L + row] : none)) / 2;
         const float need = p.need[leaf];  // the magnitude check of every element that can be non-zero
         if (!wait_acc(3)) break;
         bool bad = false;
@@ -488,6 +508,7 @@ __global__ void __launch_bounds__(kThreadsL, 1)
       }
       if (!ok) break;
       // combine: the row segment goes into every C target of the leaf
+      const int ea = F64 && row < p.L ? p.expA[(int64_t)leaf * p.L + row] : 0;
       const int nt = p.ccount[leaf];
       const CTarget* tg = p.ctab + (int64_t)leaf * p.maxT;
       unsigned long long* C = static_cast<unsigned long long*>(p.C);
@@ -499,7 +520,7 @@ __global__ void __launch_bounds__(kThreadsL, 1)
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
           // (a zero row or column has a zero sum, whatever its exponent says)
-          v[e] = F64 ? scaled_double_bits(sum[e], ea + fexp(j * 8 + e) + p.shift - 68)
+          v[e] = F64 ? scaled_double_bits(sum[e], ea + fexp(j * 8 + e) + shift - 68)
                      : (unsigned long long)sum[e];
         }
 #pragma unroll

@@ -19,6 +19,46 @@ __device__ __forceinline__ unsigned long long mag_bits(double x) {
   return (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
 }
 
+// Upper bound s 2^(2 (b - 1023)) of a sum of squares, in fp32 beside the biased
+// exponent b of an early element (the FP64 pipe does two operations a clock):
+// every element is rounded up to 21 significant bits from its high word, every
+// addition rounds up.  Elements below 2^-60 of the base count as that.
+struct SquareSum {
+  float s = 0.f;
+  int b = 0;
+  uint32_t limit = 1;  // high words from here on move the base
+
+  __device__ __forceinline__ void rebase(int to) {
+    const int e = 2 * (b - to) > -126 ? 2 * (b - to) : -126;
+    s = __fmul_ru(s, __uint_as_float((uint32_t)(127 + e) << 23));
+    b = to;
+  }
+  // before add(): `hi`, the largest high word of the elements to come
+  __device__ __forceinline__ void prepare(uint32_t hi) {
+    if (hi >= limit) {
+      rebase((int)(hi >> 20));
+      limit = (uint32_t)(b + 32) << 20;
+    }
+  }
+  __device__ __forceinline__ void add(unsigned long long mag) {
+    const int t = max((int)(uint32_t)(mag >> 32) + 1 - (b << 20), -(60 << 20));
+    const float f = __uint_as_float((uint32_t)(t + (127 << 20)) << 3);
+    s = __fmaf_ru(f, f, s);
+  }
+  __device__ __forceinline__ void merge(float s2, int b2) {
+    const int top = b > b2 ? b : b2;
+    rebase(top);
+    SquareSum o;
+    o.s = s2;
+    o.b = b2;
+    o.rebase(top);
+    s = __fadd_ru(s, o.s);
+  }
+  __device__ __forceinline__ double root() const {
+    return (double)__fsqrt_ru(s) * __hiloint2double((b > 1 ? b : 1) << 20, 0);
+  }
+};
+
 // blockIdx.z == 0: a warp takes one row of A in one column block; 1: a block
 // takes 32 columns of B in one row block.  Rows and columns beyond n are zero.
 __global__ void __launch_bounds__(256) limb_max_kernel(LimbBoundsArgs a) {
@@ -30,6 +70,7 @@ __global__ void __launch_bounds__(256) limb_max_kernel(LimbBoundsArgs a) {
     for (int64_t u = (int64_t)blockIdx.x * 8 + warp; u < a.npad * blocks; u += (int64_t)gridDim.x * 8) {
       const int64_t row = u / blocks, q = u % blocks;
       unsigned long long m = 0;
+      SquareSum sq;
       if (row < a.n) {
         const int64_t c1 = (q + 1) * L < a.n ? (q + 1) * L : a.n;
         const double* p = a.A + row * a.ld;
@@ -37,21 +78,41 @@ __global__ void __launch_bounds__(256) limb_max_kernel(LimbBoundsArgs a) {
         for (; c + 96 < c1; c += 128) {
           const unsigned long long x0 = mag_bits(p[c]), x1 = mag_bits(p[c + 32]), x2 = mag_bits(p[c + 64]),
                                    x3 = mag_bits(p[c + 96]);
-          m = max(m, max(max(x0, x1), max(x2, x3)));
+          const unsigned long long g = max(max(x0, x1), max(x2, x3));
+          m = max(m, g);
+          sq.prepare((uint32_t)(g >> 32));
+          sq.add(x0);
+          sq.add(x1);
+          sq.add(x2);
+          sq.add(x3);
         }
-        for (; c < c1; c += 32) m = max(m, mag_bits(p[c]));
+        for (; c < c1; c += 32) {
+          const unsigned long long x = mag_bits(p[c]);
+          m = max(m, x);
+          sq.prepare((uint32_t)(x >> 32));
+          sq.add(x);
+        }
       }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane == 0) a.max_a[q * a.npad + row] = __longlong_as_double((long long)m);
+      for (int o = 16; o > 0; o >>= 1) {
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        sq.merge(__shfl_xor_sync(0xffffffffu, sq.s, o), __shfl_xor_sync(0xffffffffu, sq.b, o));
+      }
+      if (lane == 0) {
+        a.max_a[q * a.npad + row] = __longlong_as_double((long long)m);
+        a.norm_a[q * a.npad + row] = sq.root();
+      }
     }
   } else {
     __shared__ unsigned long long part[8][32];
+    __shared__ float part_s[8][32];
+    __shared__ int part_b[8][32];
     const int64_t groups = a.npad / 32;
     for (int64_t u = blockIdx.x; u < groups * blocks; u += gridDim.x) {
       const int64_t col = u % groups * 32 + lane, q = u / groups;
       const int64_t r1 = (q + 1) * L < a.n ? (q + 1) * L : a.n;
       unsigned long long m = 0;
+      SquareSum sq;
       if (col < a.n) {
         const double* p = a.B + col;
         int64_t r = q * L + warp;
@@ -59,17 +120,33 @@ __global__ void __launch_bounds__(256) limb_max_kernel(LimbBoundsArgs a) {
           unsigned long long x[8];
 #pragma unroll
           for (int e = 0; e < 8; ++e) x[e] = mag_bits(p[(r + 8 * e) * a.ld]);
+          unsigned long long g = x[0];
 #pragma unroll
-          for (int e = 0; e < 8; ++e) m = max(m, x[e]);
+          for (int e = 1; e < 8; ++e) g = max(g, x[e]);
+          m = max(m, g);
+          sq.prepare((uint32_t)(g >> 32));
+#pragma unroll
+          for (int e = 0; e < 8; ++e) sq.add(x[e]);
         }
-        for (; r < r1; r += 8) m = max(m, mag_bits(p[r * a.ld]));
+        for (; r < r1; r += 8) {
+          const unsigned long long x = mag_bits(p[r * a.ld]);
+          m = max(m, x);
+          sq.prepare((uint32_t)(x >> 32));
+          sq.add(x);
+        }
       }
       part[warp][lane] = m;
+      part_s[warp][lane] = sq.s;
+      part_b[warp][lane] = sq.b;
       __syncthreads();
       if (warp == 0) {
 #pragma unroll
-        for (int w = 1; w < 8; ++w) m = max(m, part[w][lane]);
+        for (int w = 1; w < 8; ++w) {
+          m = max(m, part[w][lane]);
+          sq.merge(part_s[w][lane], part_b[w][lane]);
+        }
         a.max_b[q * a.npad + col] = __longlong_as_double((long long)m);
+        a.norm_b[q * a.npad + col] = sq.root();
       }
       __syncthreads();
     }
@@ -120,7 +197,8 @@ __global__ void __launch_bounds__(256) limb_exp_kernel(LimbBoundsArgs a, int64_t
   }
   // the divide adds level by level, the last level outermost: term u (bit k:
   // second term of level k + 1), folded pairwise from the top level down
-  double v[1 << D];
+  const double* nm = side == 0 ? a.norm_a : a.norm_b;
+  double v[1 << D], w2[1 << D];
 #pragma unroll
   for (int u = 0; u < (1 << D); ++u) {
     int64_t row = 0, col = 0;
@@ -132,16 +210,23 @@ __global__ void __launch_bounds__(256) limb_exp_kernel(LimbBoundsArgs a, int64_t
       row += (int64_t)((q >> 1) & 1) * (a.npad >> (k + 1));
       col += (int64_t)(q & 1) * (a.npad >> (k + 1));
     }
-    v[u] = 0.0;
-    if (present) v[u] = side == 0 ? mx[col / a.L * a.npad + row + i] : mx[row / a.L * a.npad + col + i];
+    v[u] = w2[u] = 0.0;
+    if (present) {
+      const int64_t at = side == 0 ? col / a.L * a.npad + row + i : row / a.L * a.npad + col + i;
+      v[u] = mx[at];
+      w2[u] = nm[at];
+    }
   }
   // S_1 sums pairs that differ in bit 0 (the top level), S_2 in bit 1, ...
 #pragma unroll
   for (int w = (1 << D) / 2; w > 0; w /= 2)
 #pragma unroll
-    for (int u = 0; u < w; ++u) v[u] = v[2 * u] + v[2 * u + 1];
+    for (int u = 0; u < w; ++u) {
+      v[u] = v[2 * u] + v[2 * u + 1];
+      w2[u] = w2[2 * u] + w2[2 * u + 1];
+    }
   const unsigned long long b = mag_bits(v[0]);
-  int32_t e = kLimbZeroRow;
+  int32_t e = kLimbZeroRow, h = a.log_l + 2;
   if (b != 0) {
     const int ex = (int)(b >> 52);
     e = ex - 1023 + ((b & 0xFFFFFFFFFFFFFull) ? 1 : 0);  // smallest e with bound <= 2^e (normal numbers)
@@ -149,8 +234,14 @@ __global__ void __launch_bounds__(256) limb_exp_kernel(LimbBoundsArgs a, int64_t
       *(volatile int*)a.flag = 1;
       e = 0;  // (any value: the product is redone)
     }
+    // N <= 2^(half / 2), from the norm's high word plus one (the sums above
+    // round to nearest); N >= R / 2, as every block's norm is at least its maximum
+    const uint32_t nh = (uint32_t)((unsigned long long)__double_as_longlong(w2[0]) >> 32) + 1u;
+    const int half = 2 * ((int)(nh >> 20) - 1023) + ((nh & 0xFFFFFu) <= 0x6A09Du ? 1 : 2);  // (0x1.6A09Ep0 <= sqrt(2))
+    h = min(max(a.log_l + 2 * e - half, 0), a.log_l + 2);
   }
   (side == 0 ? a.expA : a.expB)[t] = e;
+  (side == 0 ? a.slackA : a.slackB)[t] = h;
 }
 
 template <int D>

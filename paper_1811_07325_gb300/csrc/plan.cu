@@ -671,43 +671,34 @@ static void limb_check_sums(const stark_plan_s* p, std::vector<float>& need) {
     if (terms[(size_t)l] < kLimbCheckK) need[(size_t)l] = terms[(size_t)l] < 16 ? 0.f : (float)terms[(size_t)l];
 }
 
-// Bytes of an F64 plan's bounds, exponents, magnitude planes and flag (every
-// part a multiple of 256).
-static int64_t limb_aux_bytes(const stark_plan_s* p) {
-  const int64_t maxima = (p->npad << p->depth) * 8, exps = (p->P * p->L * 4 + 255) / 256 * 256,
-                mags = p->P * p->L * kLimbCheckK * 2, needs = (p->P * 4 + 255) / 256 * 256,
-                commons = (p->L * 4 + 255) / 256 * 256;
-  return 256 + needs + 2 * (maxima + exps + mags + commons);
+// The F64 side arrays of a plan in one allocation at `base` (null: their size
+// alone); every part is a multiple of 256 bytes.
+static int64_t limb_aux_layout(stark_plan_s* p, char* base) {
+  int64_t at = 0;
+  auto part = [&](auto*& ptr, int64_t bytes) {
+    if (base) ptr = reinterpret_cast<std::remove_reference_t<decltype(ptr)>>(base + at);
+    at += (bytes + 255) / 256 * 256;
+  };
+  const int64_t blocks = (p->npad << p->depth) * 8, rows = p->P * p->L * 4, mags = p->P * p->L * kLimbCheckK * 2;
+  part(p->d_flag, 4);
+  part(p->limb_need, p->P * 4);
+  for (int32_t** c : {&p->common_a, &p->common_b}) part(*c, p->L * 4);
+  for (int32_t** e : {&p->exp_a, &p->exp_b, &p->slack_a, &p->slack_b}) part(*e, rows);
+  for (double** m : {&p->max_a, &p->max_b, &p->norm_a, &p->norm_b}) part(*m, blocks);
+  for (void** m : {&p->mag_a, &p->mag_b}) part(*m, mags);
+  return at;
 }
 
 // What limb leaves need besides the digit planes: product planes (depth >= 1)
 // and, for F64, the side arrays.  On failure nothing new is kept.
 static bool plan_limb_extras(stark_plan_s* p) {
-  const int64_t products = p->P * p->L * p->L * 8, aux = limb_aux_bytes(p);
+  const int64_t products = p->P * p->L * p->L * 8, aux = limb_aux_layout(p, nullptr);
   const bool had_m = p->limb_m, had_aux = p->limb_aux;
   bool ok = p->depth == 0 || had_m || cudaMalloc(&p->limb_m, (size_t)products) == cudaSuccess;
   if (ok && p->dt == STARK_F64 && !had_aux) {
     ok = cudaMalloc(&p->limb_aux, (size_t)aux) == cudaSuccess;
     if (ok) {
-      const int64_t maxima = (p->npad << p->depth) * 8, exps = (p->P * p->L * 4 + 255) / 256 * 256,
-                    mags = p->P * p->L * kLimbCheckK * 2, needs = (p->P * 4 + 255) / 256 * 256,
-                    commons = (p->L * 4 + 255) / 256 * 256;
-      char* b = static_cast<char*>(p->limb_aux);
-      p->d_flag = reinterpret_cast<int*>(b);
-      b += 256;
-      p->limb_need = reinterpret_cast<float*>(b);
-      b += needs;
-      p->common_a = reinterpret_cast<int32_t*>(b);
-      p->common_b = reinterpret_cast<int32_t*>(b + commons);
-      b += 2 * commons;
-      p->mag_a = b;
-      p->mag_b = b + mags;
-      b += 2 * mags;
-      p->exp_a = reinterpret_cast<int32_t*>(b);
-      p->exp_b = reinterpret_cast<int32_t*>(b + exps);
-      b += 2 * exps;
-      p->max_a = reinterpret_cast<double*>(b);
-      p->max_b = reinterpret_cast<double*>(b + maxima);
+      limb_aux_layout(p, static_cast<char*>(p->limb_aux));
       std::vector<float> need;
       limb_check_sums(p, need);
       ok = cudaMemcpy(p->limb_need, need.data(), need.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
@@ -789,7 +780,7 @@ static void plan_free_products(stark_plan_s* p) {
   }
   if (p->limb_aux) {
     cudaFree(p->limb_aux);
-    p->ws_bytes -= limb_aux_bytes(p);
+    p->ws_bytes -= limb_aux_layout(p, nullptr);
   }
   p->int_m = p->limb_m = p->limb_aux = nullptr;
 }
@@ -1470,14 +1461,20 @@ static stark_status plan_leaves(stark_plan_s* p, void* C, int64_t lb, int64_t le
   return st;
 }
 
+static int ceil_log2(int64_t x) {
+  int l = 0;
+  while (((int64_t)1 << l) < x) ++l;
+  return l;
+}
+
 // Digit planes of every leaf operand (I64, F64), for F64 after the bounds.
 static stark_status plan_limb_divide(stark_plan_s* p, const void* A, const void* B, cudaStream_t s) {
   DivideArgs da{A, core_side(p), p->npad, p->L, p->X, nullptr, p->d_err, -1, p->n};
   DivideArgs db{B, core_side(p), p->npad, p->L, p->Y, nullptr, p->d_err, -1, p->n};
   if (p->dt == STARK_F64) {
     const LimbBoundsArgs b{static_cast<const double*>(A), static_cast<const double*>(B), core_side(p), p->n, p->npad,
-                           p->L, p->depth, p->max_a, p->max_b, p->exp_a, p->exp_b, p->common_a, p->common_b,
-                           p->d_flag};
+                           p->L, p->depth, p->max_a, p->max_b, p->norm_a, p->norm_b, p->exp_a, p->exp_b,
+                           p->slack_a, p->slack_b, ceil_log2(p->L), p->common_a, p->common_b, p->d_flag};
     if (stark_status st = to_status(launch_limb_bounds(b, s)); st != STARK_OK) return st;
     da.exps = p->exp_a;
     db.exps = p->exp_b;
@@ -1513,8 +1510,9 @@ static stark_status plan_limb_leaves(stark_plan_s* p, const void* A, const void*
   a.expB = p->exp_b;
   a.need = p->limb_need;
   a.flag = p->d_flag;
-  a.shift = 6;
-  while (((int64_t)1 << (a.shift - 6)) < p->L) ++a.shift;
+  a.slackA = p->slack_a;
+  a.slackB = p->slack_b;
+  a.shift = 6 + ceil_log2(p->L);
   stark_status st = to_status(launch_leaf_limb(a, &p->tmLA, &p->tmLB, &p->tmSA, &p->tmSB, f64, p->num_sms, s));
   if (cudaEvent_t* ev = plan_timing_events(p)) {
     cudaEventRecord(ev[3], s);  // the leaf products end

@@ -90,6 +90,10 @@ struct stark_plan_s {
   void* limb_aux = nullptr;  // F64: the arrays below, in one allocation
   double* max_a = nullptr;   // [2^depth][npad] block maxima of A's rows
   double* max_b = nullptr;   // and of B's columns
+  double* norm_a = nullptr;  // the same of 2-norms
+  double* norm_b = nullptr;
+  int32_t* slack_a = nullptr;  // [P][L] (LimbBoundsArgs::slackA)
+  int32_t* slack_b = nullptr;
   int32_t* exp_a = nullptr;  // [P][L] exponents of the leaf operands' rows
   int32_t* exp_b = nullptr;  // and columns
   int32_t* common_a = nullptr;  // [L] exponents shared by the leaves (limb_bounds.cu)

@@ -118,8 +118,13 @@ struct LimbBoundsArgs {
   int depth;
   double* max_a;      // [2^depth column blocks][npad]: row maxima of |A|
   double* max_b;      // [2^depth row blocks][npad]: column maxima of |B|
+  double* norm_a;     // the same of 2-norms, rounded up
+  double* norm_b;
   int32_t* expA;      // [7^depth][L]
   int32_t* expB;
+  int32_t* slackA;    // [7^depth][L]: how far the row's (column's) 2-norm N is below the most that R = 2^e
+  int32_t* slackB;    // allows: N <= 2^((log_l - slack) / 2) R, 0 <= slack <= log_l + 2
+  int log_l;          // 2^log_l >= L
   int32_t* common_a;  // [L]
   int32_t* common_b;
   int* flag;          // cleared, then set for infinities, NaN and exponents outside +-400
@@ -276,8 +281,11 @@ struct LeafLimbArgs {
   // F64 only
   const int32_t* expA;  // [leaf][L]: exponent e of a row of A, |x| <= 2^e (kLimbZeroRow: all zero)
   const int32_t* expB;  // [leaf][L]: the same of a column of B
+  const int32_t* slackA;  // [leaf][L] (LimbBoundsArgs)
+  const int32_t* slackB;
   const float* need;    // [leaf]: digit-magnitude sum that proves an element (limb_check_sum)
-  int32_t shift;        // the running sums' unit, 2^shift of 256^7: log2(L) rounded up, plus 6
+  int32_t shift;        // the running sums' unit where a row and its column have no slack, 2^shift
+                        // of 256^7: log2(L) rounded up, plus 6
   int* flag;            // set to 1 when an element's accuracy is not proven
 };
 cudaError_t launch_leaf_limb(const LeafLimbArgs& a, const CUtensorMap* tmA, const CUtensorMap* tmB,

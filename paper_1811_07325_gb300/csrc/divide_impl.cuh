@@ -303,7 +303,9 @@ struct Loader {
   }
   __device__ __forceinline__ Vec<Acc, VEC> operator()(int64_t row, int64_t col) const {
     Vec<Acc, VEC> r;
-    if (row < n && col + VEC <= n && vec_ok) {
+    // (a negative position is none: compared unsigned, with that of the vector's
+    // last element, as col may be -VEC)
+    if ((uint64_t)row < (uint64_t)n && (uint64_t)(col + VEC - 1) < (uint64_t)n && vec_ok) {
       const Tin* p = X + row * ld + col;
       if constexpr (sizeof(Tin) * VEC % 16 == 0) {
         constexpr int W = (int)sizeof(Tin) * VEC / 16;
@@ -320,7 +322,9 @@ struct Loader {
     } else {
 #pragma unroll
       for (int e = 0; e < VEC; ++e)
-        r.v[e] = (row < n && col + e < n) ? value(load_one(X + row * ld + col + e), e) : Acc(0);
+        r.v[e] = ((uint64_t)row < (uint64_t)n && (uint64_t)(col + e) < (uint64_t)n)
+                     ? value(load_one(X + row * ld + col + e), e)
+                     : Acc(0);
     }
     return r;
   }
@@ -407,6 +411,9 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
   const int64_t i = pos / per_row;
   const int64_t j = (pos % per_row) * VEC;
   const Loader<Tin, VEC> ld0{static_cast<const Tin*>(a.X), a.n, a.ld, vec_ok != 0};
+  // F64 digit planes: the inputs begin a.koff (even) further along K; before
+  // them the loader sees negative positions, which are zeros
+  constexpr bool kShifted = OUT == kOutLimbs && !std::is_same_v<Tin, int64_t>;
   using LoadT = std::conditional_t<(K > 0), TopLoader<Tin, VEC, SIDE, (K > 0 ? K : 1)>, Loader<Tin, VEC>>;
   LoadT ld;
   if constexpr (K > 0) {
@@ -430,7 +437,7 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
     emit.common[0] = ld.common[0];
     emit.common[1] = ld.common[1];
   }
-  if constexpr (OUT == kOutLimbs && !std::is_same_v<Tin, int64_t>) {
+  if constexpr (kShifted) {
     emit.exps = a.exps + (SIDE == 0 ? i : j);
     emit.exp_leaf = a.L;
     emit.exp_step = SIDE;
@@ -442,6 +449,7 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
       emit.mags = i < kLimbCheckK ? mags + i * a.L + j : nullptr;
   }
   const int64_t npad = a.npad;
+  const int64_t row0 = kShifted && SIDE == 1 ? i - a.koff : i, col0 = kShifted && SIDE == 0 ? j - a.koff : j;
 
   auto run_tree = [&](const Vec<Acc, VEC>(&in)[pow4c(R)], int prefix) {
     if constexpr (OUT == kOutLimbs && R == 2) {
@@ -467,7 +475,7 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
       const TermPair t = terms_of<SIDE>(dig[0]);
       const int64_t h = npad >> 1;
       auto at = [&](int g, int q) {
-        int64_t r = i + (q >> 1) * h, c = j + (q & 1) * h;
+        int64_t r = row0 + (q >> 1) * h, c = col0 + (q & 1) * h;
 #pragma unroll
         for (int k = 0; k < R; ++k) {
           const int digit = (g >> (2 * (R - 1 - k))) & 3;
@@ -490,7 +498,7 @@ __device__ __forceinline__ void divide_body(const DivideArgs& a, int vec_ok) {
     }
 #pragma unroll
     for (int g = 0; g < pow4c(R); ++g) {
-      int64_t r = i, c = j;
+      int64_t r = row0, c = col0;
 #pragma unroll
       for (int k = 0; k < R; ++k) {
         const int digit = (g >> (2 * (R - 1 - k))) & 3;

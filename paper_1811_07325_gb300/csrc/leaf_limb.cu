@@ -67,9 +67,9 @@
 // from one half, so T units are at least T / 4 / 64^2 R C:
 // T = 2^14 (2^-6 + 3/2 L / 128 2^-9) makes the digits' bound the smaller one
 // (two rounded diagonals instead of three up to L = 1024: T = 512).
-// Leaves that padding leaves with fewer than 128 terms at depth >= 1 are held
-// to one unit a term (none below 16 terms): their products enter C beside
-// full ones, whose rounding errors are larger than theirs.
+// Leaves that padding leaves with fewer than 128 terms at depth >= 1 (at least
+// 64, see limb_k_offset in plan.cu) are held to one unit a term: their products
+// enter C beside full ones, whose rounding errors are larger than theirs.
 #include <cstring>
 
 #include "leaf_common.cuh"

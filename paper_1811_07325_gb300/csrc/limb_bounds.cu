@@ -72,9 +72,10 @@ __global__ void __launch_bounds__(256) limb_max_kernel(LimbBoundsArgs a) {
       unsigned long long m = 0;
       SquareSum sq;
       if (row < a.n) {
-        const int64_t c1 = (q + 1) * L < a.n ? (q + 1) * L : a.n;
+        const int64_t c0 = q * L > a.koff ? q * L - a.koff : 0;
+        const int64_t c1 = (q + 1) * L - a.koff < a.n ? (q + 1) * L - a.koff : a.n;
         const double* p = a.A + row * a.ld;
-        int64_t c = q * L + lane;
+        int64_t c = c0 + lane;
         for (; c + 96 < c1; c += 128) {
           const unsigned long long x0 = mag_bits(p[c]), x1 = mag_bits(p[c + 32]), x2 = mag_bits(p[c + 64]),
                                    x3 = mag_bits(p[c + 96]);
@@ -110,12 +111,13 @@ __global__ void __launch_bounds__(256) limb_max_kernel(LimbBoundsArgs a) {
     const int64_t groups = a.npad / 32;
     for (int64_t u = blockIdx.x; u < groups * blocks; u += gridDim.x) {
       const int64_t col = u % groups * 32 + lane, q = u / groups;
-      const int64_t r1 = (q + 1) * L < a.n ? (q + 1) * L : a.n;
+      const int64_t r0 = q * L > a.koff ? q * L - a.koff : 0;
+      const int64_t r1 = (q + 1) * L - a.koff < a.n ? (q + 1) * L - a.koff : a.n;
       unsigned long long m = 0;
       SquareSum sq;
       if (col < a.n) {
         const double* p = a.B + col;
-        int64_t r = q * L + warp;
+        int64_t r = r0 + warp;
         for (; r + 56 < r1; r += 64) {
           unsigned long long x[8];
 #pragma unroll

@@ -644,6 +644,16 @@ static stark_status plan_tune_combine(stark_plan_t p) {
   return st;
 }
 
+// F64: the padding along K.  The last block of a leaf side that holds inputs
+// may hold only a few of them, too few terms to prove products of that block
+// alone accurate.  Where it has fewer than 64, some of the zeros go ahead of the
+// inputs instead of after them, so that the last block and the first 128 of the
+// first one have at least 64 each.
+static int64_t limb_k_offset(int64_t n, int64_t L, int depth) {
+  const int64_t last = n > 0 ? (n - 1) % L + 1 : L;  // inputs in the last block
+  return depth == 0 || last >= 64 ? 0 : ((129 - last) / 2 + 1) / 2 * 2;
+}
+
 // The magnitude sum each F64 leaf's elements must reach (leaf_limb.cu has the
 // derivation), from the leaf side and the terms that padding leaves the leaf.
 static void limb_check_sums(const stark_plan_s* p, std::vector<float>& need) {
@@ -652,23 +662,29 @@ static void limb_check_sums(const stark_plan_s* p, std::vector<float>& need) {
   const float full_need = (float)std::max(512.0, full);
   need.assign((size_t)p->P, full_need);
   if (p->depth == 0) return;
-  std::vector<int64_t> terms((size_t)p->P, kLimbCheckK);
+  // K positions [first, last) with an input element in some term, on both sides
+  std::vector<int64_t> first((size_t)p->P, 0), last((size_t)p->P, p->L);
   for (int side = 0; side < 2; ++side) {
     std::vector<int32_t> cnt, quad;
     std::vector<int8_t> sign;
     build_quadrant_table(p->depth, side, cnt, quad, sign);
     for (int64_t l = 0; l < p->P; ++l) {
-      int64_t k = 0;  // K positions with an input element in some term (columns of A, rows of B)
+      int64_t k0 = p->L, k1 = 0;  // (the union is an interval)
       for (int t = 0; t < cnt[(size_t)l]; ++t) {
         int64_t r = 0, c = 0;
         quadrant_offsets(p->depth, p->npad, quad[(size_t)(l << p->depth) + t], &r, &c);
-        k = std::max(k, core_side(p) - (side == 0 ? c : r));
+        const int64_t at = side == 0 ? c : r;  // columns of A, rows of B
+        k0 = std::min(k0, std::max<int64_t>(0, p->koff - at));
+        k1 = std::max(k1, std::min(p->L, p->koff + core_side(p) - at));
       }
-      terms[(size_t)l] = std::min(terms[(size_t)l], k);
+      first[(size_t)l] = std::max(first[(size_t)l], k0);
+      last[(size_t)l] = std::min(last[(size_t)l], k1);
     }
   }
-  for (int64_t l = 0; l < p->P; ++l)
-    if (terms[(size_t)l] < kLimbCheckK) need[(size_t)l] = terms[(size_t)l] < 16 ? 0.f : (float)terms[(size_t)l];
+  for (int64_t l = 0; l < p->P; ++l) {
+    const int64_t terms = std::min<int64_t>(last[(size_t)l], kLimbCheckK) - first[(size_t)l];
+    if (terms < kLimbCheckK) need[(size_t)l] = (float)std::max<int64_t>(terms, 0);
+  }
 }
 
 // The F64 side arrays of a plan in one allocation at `base` (null: their size
@@ -699,6 +715,7 @@ static bool plan_limb_extras(stark_plan_s* p) {
     ok = cudaMalloc(&p->limb_aux, (size_t)aux) == cudaSuccess;
     if (ok) {
       limb_aux_layout(p, static_cast<char*>(p->limb_aux));
+      p->koff = limb_k_offset(core_side(p), p->L, p->depth);
       std::vector<float> need;
       limb_check_sums(p, need);
       ok = cudaMemcpy(p->limb_need, need.data(), need.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
@@ -1474,7 +1491,7 @@ static stark_status plan_limb_divide(stark_plan_s* p, const void* A, const void*
   if (p->dt == STARK_F64) {
     const LimbBoundsArgs b{static_cast<const double*>(A), static_cast<const double*>(B), core_side(p), p->n, p->npad,
                            p->L, p->depth, p->max_a, p->max_b, p->norm_a, p->norm_b, p->exp_a, p->exp_b,
-                           p->slack_a, p->slack_b, ceil_log2(p->L), p->common_a, p->common_b, p->d_flag};
+                           p->slack_a, p->slack_b, ceil_log2(p->L), p->koff, p->common_a, p->common_b, p->d_flag};
     if (stark_status st = to_status(launch_limb_bounds(b, s)); st != STARK_OK) return st;
     da.exps = p->exp_a;
     db.exps = p->exp_b;
@@ -1482,6 +1499,7 @@ static stark_status plan_limb_divide(stark_plan_s* p, const void* A, const void*
     db.common = p->common_b;
     da.mags = p->mag_a;
     db.mags = p->mag_b;
+    da.koff = db.koff = p->koff;
   }
   return to_status(launch_divide_limbs(da, db, p->depth, p->dt == STARK_F64 ? kInF64 : kInI64, s));
 }

@@ -88,6 +88,7 @@ struct DivideArgs {
   // kLimbZeroRow where they differ too much (limb_bounds.cu)
   const int32_t* common;
   void* mags;
+  int64_t koff;  // even: zeros ahead of the inputs along K (columns of A, rows of B); koff + n <= npad
 };
 
 // Divide phase for one operand: writes the 7^depth leaf operand sums as
@@ -125,6 +126,7 @@ struct LimbBoundsArgs {
   int32_t* slackA;    // [7^depth][L]: how far the row's (column's) 2-norm N is below the most that R = 2^e
   int32_t* slackB;    // allows: N <= 2^((log_l - slack) / 2) R, 0 <= slack <= log_l + 2
   int log_l;          // 2^log_l >= L
+  int64_t koff;       // zeros ahead of the inputs along K
   int32_t* common_a;  // [L]
   int32_t* common_b;
   int* flag;          // cleared, then set for infinities, NaN and exponents outside +-400

@@ -15,7 +15,7 @@ namespace {
 // instead of 512 us at n = 4096, depth 2.
 template <typename Tin, int D, int SIDE>
 __device__ __forceinline__ void limb_body(const DivideArgs& a, int vec) {
-  if constexpr (std::is_same_v<Tin, double>) {
+  if constexpr (std::is_same_v<Tin, double> && D <= kLimbFixedDepth) {
     const int64_t pos = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, per_row = a.L / 2;
     if (pos >= a.L * per_row) return;
     const int64_t i = pos / per_row, j = pos % per_row * 2;

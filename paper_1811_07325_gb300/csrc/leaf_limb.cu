@@ -42,34 +42,47 @@
 // steps, the issuing thread needed 760 cycles a step on its own and the
 // kernel ran at 30 % of the fp16 rate (6.5 ms for 49 leaves of side 1024).
 //
-// F64 accuracy.  The operands are sums of up to 2^d inputs: an fp64 sum rounded
-// to 2^-62 of the row's bound R (a power of two), or an integer sum off by at
-// most 2^(d+2) such units (limb_bounds.cu), 2^-57 R at depth 3, where the fp64
-// sums alone are off by 2^-53 of themselves a level.  Given them, and with C
-// the bound of the column of B, a product of K non-zero terms is off by at most K 2^-59 R C (the dropped digit products,
-// 7 * 2^14 * 256^6 / 2^124 a term) and half a unit of the running sum for
-// every rounded diagonal.  The sum keeps 64 bits, so the unit follows from the
-// most that the product can be: by Cauchy and Schwarz at most the product of
-// the 2-norms of its row and column, which limb_bounds.cu has as R C 2^l
-// (2^l >= L) less the slacks of both.  With the slack of its own row and the
-// least of its warp's 64 columns, the unit is 2^(l - 62) R C less that: at most
-// 2^-59 of those norms' product unless a column stands out among the 64.  (With
-// the unit 2^(l - 62) R C of rows without slack, rows of 1024 elements of about
-// one with a single one of up to 32 were off by 5 times as much as in FP64.)
-// A K-term FP64 dot product is
-// only bound to K 2^-53 sum |a||b|.  So the digits are the more accurate of
-// the two unless nearly every |a||b| is far below R C (badly scaled or sparse
-// rows), and the kernel proves for each element that it is not: over the
-// first 128 of K the digit products of magnitudes, sum |a_0||b_0|, must reach
-// need[leaf], else it raises `flag` and the product is redone on the CUDA
-// cores (as for infinities, NaN and exponents outside +-400, flagged by the
-// bounds kernel).  A magnitude digit is 64 at the bound and may be rounded up
-// from one half, so T units are at least T / 4 / 64^2 R C:
-// T = 2^14 (2^-6 + 3/2 L / 128 2^-9) makes the digits' bound the smaller one
-// (two rounded diagonals instead of three up to L = 1024: T = 512).
-// Leaves that padding leaves with fewer than 128 terms at depth >= 1 (at least
-// 64, see limb_k_offset in plan.cu) are held to one unit a term: their products
-// enter C beside full ones, whose rounding errors are larger than theirs.
+// F64 accuracy.  R and C are the powers of two that bound a row of the left
+// operand and a column of the right one, k the terms that are not padding and u
+// 2^-53.  A k-term FP64 dot product is bound to k u sum |a||b|; against the exact
+// product of its operands the digits' is off by at most
+//   drop     k 7.03 2^-62 R C: the digit products below 256^7, 7 of up to 2^14 at
+//            256^6, 6 at 256^5, ...;
+//   operand  for operand elements off by eps R (eps C), eps (R sum |b| +
+//            C sum |a|), where sum |b| <= sqrt(k) times b's 2-norm.  An fp64 sum
+//            is rounded to a digit unit, eps = 2^-63; an integer sum (depths 1 to
+//            3, limb_bounds.cu) is off by up to eps = 2^(depth - 60);
+//   sum      half a unit of the running sum for every diagonal that is rounded
+//            to it, two or three in 128 of K.  The sum keeps 64 bits, so its unit
+//            follows from the most that the product can be: by Cauchy and Schwarz
+//            at most the product of the 2-norms of its row and column, which
+//            limb_bounds.cu has as R C 2^l (2^l >= L) less the slacks of both.
+//            With the slack of its own row and the least of its warp's 64
+//            columns, the unit is 2^(l - 62) R C less that: at most 2^-60 of
+//            those bounds' product unless a column stands out among the 64.
+//            (With the unit of rows without slack, rows of 1024 elements of about
+//            one with a single one of up to 32 were off by 5 times as much as
+//            in FP64.)
+// and by one rounding of the result, u sum |a||b|, of FP64's k.  So the digits
+// keep FP64's bound unless nearly every |a||b| is far below R C (badly scaled
+// or sparse rows), and the kernel proves for each element that it is not: over
+// the first 128 of K the digit products of magnitudes, sum |a_0||b_0|, must reach
+// LimbNeed, else it raises `flag` and the product is redone on the CUDA cores
+// (as for infinities, NaN and exponents outside +-400, flagged by the bounds
+// kernel).  A magnitude digit is 64 at the bound and may be rounded up from one
+// half, so T units are at least T / 4 / 64^2 R C of sum |a||b|, and the three
+// errors ask for 225, 2^14 eps / u (...) and 16 a rounded diagonal (plan.cu; 1 %
+// is for the digit's half and a bit, k / (k - 1) for the result's rounding).
+// These are bounds.  The errors themselves are an order of magnitude below
+// FP64's on data without structure (tests/test_gpu_f64_accuracy.py).  The worst
+// kind met is entries whose bits end at the top bit of a digit, 31 to 33 bits
+// below R: that digit is -128 or 0, and the dropped products add up, 2^-64 R C a
+// term.  At 512 units that was 1.07 times FP64's error; kLimbLeast is 640.
+// Padding leaves every leaf at least 64 terms to prove it by (limb_k_offset in
+// plan.cu).
+//
+// Splitting operands so that slices multiply without rounding, and summing the
+// slices' products, is Ozaki's scheme (Ozaki, Ogita, Oishi and Rump 2012).
 #include <cstring>
 
 #include "leaf_common.cuh"
@@ -477,8 +490,12 @@ __global__ void __launch_bounds__(kThreadsL, 1)
         }
         __syncwarp();
         slack = __reduce_min_sync(0xffffffffu, slack);
-        shift = p.shift - (slack + (row < p.L ? p.slackA[(int64_t)leaf * p.L + row] : none)) / 2;
-        const float need = p.need[leaf];  // the magnitude check of every element that can be non-zero
+        const int slack_a = row < p.L ? p.slackA[(int64_t)leaf * p.L + row] : none;
+        shift = p.shift - (slack + slack_a) / 2;
+        // the magnitude check of every element that can be non-zero
+        const LimbNeed q = p.need[leaf];
+        const float need = fmaxf(kLimbLeast, q.drop + q.operand * (exp2f(-0.5f * slack_a) + exp2f(-0.5f * slack)) +
+                                                 q.sum * exp2f((float)(shift - p.shift)));
         if (!wait_acc(3)) break;
         bool bad = false;
 #pragma unroll 1

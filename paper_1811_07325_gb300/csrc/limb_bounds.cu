@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(256) limb_max_kernel(LimbBoundsArgs a) {
 // lie within a factor of four, all are turned to integers by one exponent
 // ec = e(largest) + D, the operand sums are integer sums, and a leaf's digits
 // are the sum shifted by ec - e(leaf): off by at most 2^(D + 2) of the 2^-62 R
-// units per term, still 2^-57 R, where an fp64 sum is rounded to 2^-53.
+// units per term, still 2^-57 R at depth 3, where an fp64 sum is rounded to
+// 2^-53 (not at depth 4, where the check would allow twice as much for it).
 template <int D>
 __global__ void __launch_bounds__(256) limb_exp_kernel(LimbBoundsArgs a, int64_t leaves) {
   const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
@@ -182,7 +183,7 @@ __global__ void __launch_bounds__(256) limb_exp_kernel(LimbBoundsArgs a, int64_t
     const int ex = (int)(mx >> 52);
     int32_t ec = mx == 0 ? 0 : ex - 1023 + ((mx & 0xFFFFFFFFFFFFFull) ? 1 : 0) + D;
     // (magnitude bits: two exponents apart is a factor of four)
-    if (mx != 0 && (ex == 2047 || ex < 8 || mn + (2ull << 52) < mx)) ec = kLimbZeroRow;
+    if (D > kLimbFixedDepth || (mx != 0 && (ex == 2047 || ex < 8 || mn + (2ull << 52) < mx))) ec = kLimbZeroRow;
     (side == 0 ? a.common_a : a.common_b)[t] = ec;
     return;
   }

@@ -654,14 +654,17 @@ static int64_t limb_k_offset(int64_t n, int64_t L, int depth) {
   return depth == 0 || last >= 64 ? 0 : ((129 - last) / 2 + 1) / 2 * 2;
 }
 
-// The magnitude sum each F64 leaf's elements must reach (leaf_limb.cu has the
-// derivation), from the leaf side and the terms that padding leaves the leaf.
-static void limb_check_sums(const stark_plan_s* p, std::vector<float>& need) {
-  const double rounded = p->L <= 1024 ? 1.0 : 1.5;  // half units a superchunk
-  const double full = 16384.0 * (1.0 / 64 + rounded * (double)p->L / 128.0 / 512.0);
-  const float full_need = (float)std::max(512.0, full);
-  need.assign((size_t)p->P, full_need);
-  if (p->depth == 0) return;
+static int ceil_log2(int64_t x) {
+  int l = 0;
+  while (((int64_t)1 << l) < x) ++l;
+  return l;
+}
+
+// The parts of the magnitude sum each F64 leaf's elements must reach
+// (leaf_limb.cu has the derivation), from the leaf side and the terms that
+// padding leaves the leaf.
+static void limb_check_sums(const stark_plan_s* p, std::vector<LimbNeed>& need) {
+  const int l = ceil_log2(p->L);
   // K positions [first, last) with an input element in some term, on both sides
   std::vector<int64_t> first((size_t)p->P, 0), last((size_t)p->P, p->L);
   for (int side = 0; side < 2; ++side) {
@@ -681,9 +684,23 @@ static void limb_check_sums(const stark_plan_s* p, std::vector<float>& need) {
       last[(size_t)l] = std::min(last[(size_t)l], k1);
     }
   }
-  for (int64_t l = 0; l < p->P; ++l) {
-    const int64_t terms = std::min<int64_t>(last[(size_t)l], kLimbCheckK) - first[(size_t)l];
-    if (terms < kLimbCheckK) need[(size_t)l] = (float)std::max<int64_t>(terms, 0);
+  need.assign((size_t)p->P, LimbNeed{0.f, 0.f, 0.f, 0.f});
+  for (int64_t i = 0; i < p->P; ++i) {
+    const int64_t k0 = first[(size_t)i], k1 = last[(size_t)i], k = k1 - k0;
+    if (k <= 1) continue;  // (no terms: zeros)
+    // diagonals that may be rounded: above 256^4 once in 128 of K, else in 256
+    int64_t rounded = 0;
+    for (int s = 0; s < 8; ++s)
+      if (8 * (7 - s) < 6 + l) {
+        const int64_t step = s >= 4 ? 128 : 256;
+        rounded += (k1 - 1) / step - k0 / step + 1;
+      }
+    const double scale = 1.01 * (double)k / (double)(k - 1), side = std::ldexp(1.0, l) / (double)k;
+    const double operand = p->depth >= 1 && p->depth <= kLimbFixedDepth ? std::ldexp(1.0, p->depth + 7) : 16.0;
+    LimbNeed& q = need[(size_t)i];
+    q.drop = (float)(scale * 225.0);
+    q.operand = (float)(scale * operand * std::sqrt(side));
+    q.sum = (float)(scale * 16.0 * (double)rounded * side);
   }
 }
 
@@ -697,7 +714,7 @@ static int64_t limb_aux_layout(stark_plan_s* p, char* base) {
   };
   const int64_t blocks = (p->npad << p->depth) * 8, rows = p->P * p->L * 4, mags = p->P * p->L * kLimbCheckK * 2;
   part(p->d_flag, 4);
-  part(p->limb_need, p->P * 4);
+  part(p->limb_need, p->P * (int64_t)sizeof(LimbNeed));
   for (int32_t** c : {&p->common_a, &p->common_b}) part(*c, p->L * 4);
   for (int32_t** e : {&p->exp_a, &p->exp_b, &p->slack_a, &p->slack_b}) part(*e, rows);
   for (double** m : {&p->max_a, &p->max_b, &p->norm_a, &p->norm_b}) part(*m, blocks);
@@ -716,9 +733,9 @@ static bool plan_limb_extras(stark_plan_s* p) {
     if (ok) {
       limb_aux_layout(p, static_cast<char*>(p->limb_aux));
       p->koff = limb_k_offset(core_side(p), p->L, p->depth);
-      std::vector<float> need;
+      std::vector<LimbNeed> need;
       limb_check_sums(p, need);
-      ok = cudaMemcpy(p->limb_need, need.data(), need.size() * sizeof(float), cudaMemcpyHostToDevice) == cudaSuccess;
+      ok = cudaMemcpy(p->limb_need, need.data(), need.size() * sizeof(LimbNeed), cudaMemcpyHostToDevice) == cudaSuccess;
     }
   }
   if (!ok) {
@@ -1476,12 +1493,6 @@ static stark_status plan_leaves(stark_plan_s* p, void* C, int64_t lb, int64_t le
     st = to_status(p->dt == STARK_F64 ? launch_leaf_f64(a, s) : launch_leaf_i64(a, s));
   }
   return st;
-}
-
-static int ceil_log2(int64_t x) {
-  int l = 0;
-  while (((int64_t)1 << l) < x) ++l;
-  return l;
 }
 
 // Digit planes of every leaf operand (I64, F64), for F64 after the bounds.

@@ -100,7 +100,7 @@ struct stark_plan_s {
   int32_t* common_b = nullptr;
   void* mag_a = nullptr;     // [P][L][128] magnitudes of the leading digits
   void* mag_b = nullptr;     // [P][128][L]
-  float* limb_need = nullptr;  // [P] magnitude sums that prove a leaf's elements
+  stark::LimbNeed* limb_need = nullptr;  // [P] what proves a leaf's elements
   int64_t koff = 0;          // zeros ahead of the inputs along K (limb_k_offset)
   int* d_flag = nullptr;     // set when the product must be redone on the CUDA cores
   CUtensorMap tmA;

@@ -268,6 +268,14 @@ cudaError_t launch_leaf_i64(const LeafCcArgs& a, cudaStream_t s);
 // L >= 128 a multiple of 64.
 constexpr int32_t kLimbZeroRow = INT32_MIN;  // exponent of an operand row (column) that is zero
 constexpr int kLimbCheckK = 128;             // K of the F64 magnitude check's planes
+// The digit-magnitude sum that proves an element of a leaf accurate, for slacks
+// a and b of its row and column (leaf_limb.cu has the derivation):
+//   max(kLimbLeast, drop + operand (2^(-a / 2) + 2^(-b / 2)) + sum 2^-floor((a + b) / 2)).
+struct LimbNeed {
+  float drop, operand, sum, unused;
+};
+constexpr float kLimbLeast = 640.f;
+constexpr int kLimbFixedDepth = 3;  // up to here F64 operand sums may be integer sums (limb_bounds.cu)
 struct LeafLimbArgs {
   int32_t L, leaf_begin, leaf_end;
   const CTarget* ctab;
@@ -285,7 +293,7 @@ struct LeafLimbArgs {
   const int32_t* expB;  // [leaf][L]: the same of a column of B
   const int32_t* slackA;  // [leaf][L] (LimbBoundsArgs)
   const int32_t* slackB;
-  const float* need;    // [leaf]: digit-magnitude sum that proves an element (limb_check_sum)
+  const LimbNeed* need;  // [leaf]
   int32_t shift;        // the running sums' unit where a row and its column have no slack, 2^shift
                         // of 256^7: log2(L) rounded up, plus 6
   int* flag;            // set to 1 when an element's accuracy is not proven

@@ -56,8 +56,10 @@ __device__ __forceinline__ void fold(const V (&m)[7], V (&c)[4]) {
 // product (blockIdx.y) D levels up: 7^D vectors in, 4^D out.
 template <typename T, typename TM, int D, int W>
 __global__ void __launch_bounds__(256, W == 1 ? 4 : 2)
-    combine_limb_kernel(const TM* __restrict__ M, int64_t L, T* __restrict__ out, int64_t out_plane, int64_t ld, int64_t n) {
+    combine_limb_kernel(const TM* __restrict__ M, int64_t L, T* __restrict__ out, int64_t out_plane, int64_t ld, int64_t n,
+                        const int* __restrict__ skip) {
   using V = Cols<T, W>;
+  if (skip && *skip != 0) return;
   const int64_t pos = (int64_t)blockIdx.x * 256 + threadIdx.x;
   if (pos >= L * (L / W)) return;
   const int64_t r = pos / (L / W), c = pos % (L / W) * W;
@@ -131,32 +133,33 @@ __global__ void __launch_bounds__(256, W == 1 ? 4 : 2)
 
 template <typename T, int D, typename TM>
 cudaError_t fold_levels(const TM* M, int64_t L, int64_t products, T* out, int64_t out_plane, int64_t ld, int64_t n,
-                        cudaStream_t st) {
+                        const int* skip, cudaStream_t st) {
   constexpr int W = std::is_same_v<TM, double> && D == 2 ? 1 : 2;
   const int64_t blocks = (L * (L / W) + 255) / 256;
   if (L % 2 != 0 || blocks > 0x7FFFFFFF || products > 65535) return cudaErrorInvalidValue;
-  combine_limb_kernel<T, TM, D, W><<<dim3((unsigned)blocks, (unsigned)products), 256, 0, st>>>(M, L, out, out_plane, ld, n);
+  combine_limb_kernel<T, TM, D, W><<<dim3((unsigned)blocks, (unsigned)products), 256, 0, st>>>(M, L, out, out_plane, ld, n, skip);
   count_launch();
   return cudaGetLastError();
 }
 
 template <typename T, typename TM>
-cudaError_t by_depth(const void* Mv, int depth, int64_t L, int64_t n, void* Cv, int64_t ldc, void* tmp, cudaStream_t st) {
+cudaError_t by_depth(const void* Mv, int depth, int64_t L, int64_t n, void* Cv, int64_t ldc, void* tmp, const int* skip,
+                     cudaStream_t st) {
   const TM* M = static_cast<const TM*>(Mv);
   T* C = static_cast<T*>(Cv);
   T* mid = static_cast<T*>(tmp);
   const int64_t side = 4 * L;
   cudaError_t e;
   switch (depth) {
-    case 0: return fold_levels<T, 0>(M, L, 1, C, 0, ldc, n, st);
-    case 1: return fold_levels<T, 1>(M, L, 1, C, 0, ldc, n, st);
-    case 2: return fold_levels<T, 2>(M, L, 1, C, 0, ldc, n, st);
+    case 0: return fold_levels<T, 0>(M, L, 1, C, 0, ldc, n, skip, st);
+    case 1: return fold_levels<T, 1>(M, L, 1, C, 0, ldc, n, skip, st);
+    case 2: return fold_levels<T, 2>(M, L, 1, C, 0, ldc, n, skip, st);
     case 3:
-      e = fold_levels<T, 2>(M, L, 7, mid, side * side, side, side, st);
-      return e != cudaSuccess ? e : fold_levels<T, 1>(static_cast<const T*>(mid), side, 1, C, 0, ldc, n, st);
+      e = fold_levels<T, 2>(M, L, 7, mid, side * side, side, side, skip, st);
+      return e != cudaSuccess ? e : fold_levels<T, 1>(static_cast<const T*>(mid), side, 1, C, 0, ldc, n, skip, st);
     case 4:
-      e = fold_levels<T, 2>(M, L, 49, mid, side * side, side, side, st);
-      return e != cudaSuccess ? e : fold_levels<T, 2>(static_cast<const T*>(mid), side, 1, C, 0, ldc, n, st);
+      e = fold_levels<T, 2>(M, L, 49, mid, side * side, side, side, skip, st);
+      return e != cudaSuccess ? e : fold_levels<T, 2>(static_cast<const T*>(mid), side, 1, C, 0, ldc, n, skip, st);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -164,11 +167,11 @@ cudaError_t by_depth(const void* Mv, int depth, int64_t L, int64_t n, void* Cv, 
 }  // namespace
 
 cudaError_t launch_combine_limb(const void* M, int depth, int64_t L, int64_t n, void* C, int64_t ldc, void* tmp,
-                                InType t, cudaStream_t st) {
+                                InType t, const int* skip, cudaStream_t st) {
   switch (t) {
-    case kInF64: return by_depth<double, double>(M, depth, L, n, C, ldc, tmp, st);
-    case kInI64: return by_depth<unsigned long long, unsigned long long>(M, depth, L, n, C, ldc, tmp, st);
-    default: return by_depth<unsigned long long, float>(M, depth, L, n, C, ldc, tmp, st);
+    case kInF64: return by_depth<double, double>(M, depth, L, n, C, ldc, tmp, skip, st);
+    case kInI64: return by_depth<unsigned long long, unsigned long long>(M, depth, L, n, C, ldc, tmp, skip, st);
+    default: return by_depth<unsigned long long, float>(M, depth, L, n, C, ldc, tmp, skip, st);
   }
 }
 

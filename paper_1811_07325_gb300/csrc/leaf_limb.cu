@@ -141,6 +141,9 @@ __global__ void __launch_bounds__(kThreadsL, 1)
   auto accf_bar = [&](int a) { return bar_base + 8 * (2 * kQuads + a); };
   auto acce_bar = [&](int a) { return bar_base + 8 * (2 * kQuads + 4 + a); };
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kQuads * kQuadBytes + kEpiBytes + 8 * (2 * kQuads + 8));
+  // F64: set by the producer, ahead of the barrier of a tile's first quad, once
+  // the product's flag is up: the product is redone, and no role goes on
+  volatile int* stop = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x / 32;
   const int lane = threadIdx.x % 32;
@@ -151,6 +154,7 @@ __global__ void __launch_bounds__(kThreadsL, 1)
   const int chunks = (kblocks + 3) / 4;  // 128 of K each, the last one possibly 64
 
   if (threadIdx.x == 0) {
+    *stop = 0;
     for (int s = 0; s < kQuads; ++s) {
       mbar_init(full_bar(s), 1);
       mbar_init(empty_bar(s), 1);
@@ -215,6 +219,15 @@ __global__ void __launch_bounds__(kThreadsL, 1)
         const int leaf = p.leaf_begin + item / per_leaf;  // workspace plane
         const int tile = item % per_leaf;
         const int m0 = tile / tiles * 128, n0 = tile % tiles * 128;
+        if (F64 && *(volatile const int*)p.flag != 0) {
+          if (!mbar_wait_bounded(empty_bar(slot), phase ^ 1, p.err, kDevTimeoutEmpty, p.timeout_ns)) {
+            ok = false;
+          } else {
+            *stop = 1;
+            mbar_arrive(full_bar(slot));
+          }
+          break;
+        }
         if (F64) {
           // magnitudes: the four K blocks of 32 take the place of the digits
           uint32_t st = next();
@@ -380,9 +393,17 @@ __global__ void __launch_bounds__(kThreadsL, 1)
         mma_commit(empty_bar(sb));
         return true;
       };
-      auto check = [&]() -> bool {
+      // the magnitude products; `go_on` false: the product is redone
+      auto check = [&](bool& go_on) -> bool {
         int sa, sb;
-        if ((sa = take()) < 0 || (sb = take()) < 0 || !wait_free(3)) return false;
+        if ((sa = take()) < 0) return false;
+        if (*stop) {
+          go_on = false;
+          if (!wait_free(3)) return false;
+          mbar_arrive(accf_bar(3));  // (in place of the MMAs' commit)
+          return true;
+        }
+        if ((sb = take()) < 0 || !wait_free(3)) return false;
         tc_fence_after();
         const uint32_t a = lo_a(sa), b = lo_b(sb);
 #pragma unroll
@@ -393,7 +414,11 @@ __global__ void __launch_bounds__(kThreadsL, 1)
         return true;
       };
       for (int item = blockIdx.x; ok && item < num_items; item += gridDim.x) {
-        if (F64) ok = check();
+        if (F64) {
+          bool go_on = true;
+          ok = check(go_on);
+          if (!go_on) break;
+        }
         for (int b0 = 0; ok && b0 < kblocks; b0 += 8) {
           const int b1 = b0 + 8 < kblocks ? b0 + 8 : kblocks;
           issued = true;
@@ -496,7 +521,7 @@ __global__ void __launch_bounds__(kThreadsL, 1)
         const LimbNeed q = p.need[leaf];
         const float need = fmaxf(kLimbLeast, q.drop + q.operand * (exp2f(-0.5f * slack_a) + exp2f(-0.5f * slack)) +
                                                  q.sum * exp2f((float)(shift - p.shift)));
-        if (!wait_acc(3)) break;
+        if (!wait_acc(3) || *stop) break;
         bool bad = false;
 #pragma unroll 1
         for (int j = 0; j < 4; ++j) {

@@ -1473,7 +1473,7 @@ static stark_status plan_leaves(stark_plan_s* p, void* C, int64_t lb, int64_t le
         cudaEventRecord(ev[3], s);  // the leaf products end, the combine pass starts
         p->timing_leaf_marked = true;
       }
-      st = to_status(launch_combine_limb(p->int_m, p->depth, p->L, core_side(p), C, p->n, p->X, kInF32, s));
+      st = to_status(launch_combine_limb(p->int_m, p->depth, p->L, core_side(p), C, p->n, p->X, kInF32, nullptr, s));
     }
   } else {
     LeafCcArgs a{};
@@ -1549,7 +1549,7 @@ static stark_status plan_limb_leaves(stark_plan_s* p, const void* A, const void*
   }
   if (st == STARK_OK && stored && p->depth > 0)
     st = to_status(launch_combine_limb(p->limb_m, p->depth, p->L, core_side(p), C, p->n, p->X,
-                                       f64 ? kInF64 : kInI64, s));
+                                       f64 ? kInF64 : kInI64, f64 ? p->d_flag : nullptr, s));
   if (st != STARK_OK || !f64) return st;
   DivideArgs da{A, core_side(p), p->npad, p->L, p->X, nullptr, p->d_err, -1, p->n};
   DivideArgs db{B, core_side(p), p->npad, p->L, p->Y, nullptr, p->d_err, -1, p->n};

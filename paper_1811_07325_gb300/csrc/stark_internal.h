@@ -296,7 +296,7 @@ struct LeafLimbArgs {
   const LimbNeed* need;  // [leaf]
   int32_t shift;        // the running sums' unit where a row and its column have no slack, 2^shift
                         // of 256^7: log2(L) rounded up, plus 6
-  int* flag;            // set to 1 when an element's accuracy is not proven
+  int* flag;            // set to 1 when an element's accuracy is not proven; tiles begun after that are left out
 };
 cudaError_t launch_leaf_limb(const LeafLimbArgs& a, const CUtensorMap* tmA, const CUtensorMap* tmB,
                              const CUtensorMap* tmSA, const CUtensorMap* tmSB, bool f64, int num_sms,
@@ -305,9 +305,9 @@ cudaError_t launch_leaf_limb(const LeafLimbArgs& a, const CUtensorMap* tmA, cons
 // Ordered combine of stored leaf products M [7^depth][L][L] into a C of 8-byte
 // elements (depth 0..4): fp64 (kInF64), int64 (kInI64), or integers held in
 // fp32 into int64 (kInF32).  tmp: 7^(depth - 2) (4 L)^2 elements of C's type
-// for depths 3 and 4.
+// for depths 3 and 4.  skip not null: nothing is done where *skip != 0.
 cudaError_t launch_combine_limb(const void* M, int depth, int64_t L, int64_t n, void* C, int64_t ldc, void* tmp,
-                                InType t, cudaStream_t s);
+                                InType t, const int* skip, cudaStream_t s);
 
 cudaError_t launch_wait_selftest(int* err, uint64_t timeout_ns, cudaStream_t s);
 

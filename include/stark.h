@@ -86,7 +86,7 @@ typedef struct {
   int32_t dtype;           /* stark_dtype                                                 */
   int64_t leaves;          /* 7^depth                                                    */
   int64_t workspace_bytes; /* device bytes the plan owns (leaf operands, tables, ...)    */
-  int32_t tile_m, tile_n;  /* leaf GEMM output tile                                      */
+  int32_t tile_m, tile_n;  /* leaf GEMM output tile of a whole product                   */
   int32_t peel;            /* edge rows/columns done classically (STARK_PLAN_PEEL), else 0 */
   int32_t combine;         /* combine mode in effect (stark_plan_set_combine)            */
   int32_t shard_levels;    /* stark_plan_set_shard: top levels above the shard's subtrees (0: none) */

@@ -261,6 +261,8 @@ static bool plan_limbs(const stark_plan_s* p) {
          (p->dt != STARK_F64 || p->limb_aux);
 }
 
+static bool plan_narrow(const stark_plan_s* p, int64_t lb, int64_t le);
+
 // Tensor maps of the digit planes.
 static bool plan_limb_maps(stark_plan_s* p) {
   // A: four planes of 128 rows x 32 of K; B: four of 32 of K x 64 columns
@@ -406,7 +408,7 @@ stark_status stark_plan_get_info(stark_plan_t p, stark_plan_info* info) {
   info->workspace_bytes = p->ws_bytes;
   const bool limbs = plan_limbs(p);
   info->tile_m = p->is_tc || limbs ? 128 : 64;
-  info->tile_n = p->is_tc ? p->bn : limbs ? 128 : 64;
+  info->tile_n = p->is_tc ? (plan_narrow(p, 0, p->P) ? 128 : p->bn) : limbs ? 128 : 64;
   info->combine = p->combine_mode;
   info->shard_levels = p->shard_levels;
   info->shard_first = (int32_t)p->shard_first;

@@ -117,8 +117,8 @@ cudaError_t launch(const LeafCcArgs& a, cudaStream_t st) {
   if (leaves > 65535 || a.L / BT > 65535) return cudaErrorInvalidValue;
   const int64_t items = (int64_t)leaves * (a.L / BT) * (a.L / BT);
   // one tile per block; a gated launch, which usually does nothing, has only
-  // as many blocks as run at once (351,232 tiles would take 0.2 ms to skip)
-  const int64_t limit = a.gate ? 8 * 152 : 0x7FFFFFFF;
+  // eight blocks an SM (351,232 tiles would take 0.2 ms to skip)
+  const int64_t limit = a.gate ? 8 * device_sm_count() : 0x7FFFFFFF;
   leaf_cc_kernel<T><<<(unsigned)(items < limit ? items : limit), 256, 0, st>>>(a);
   count_launch();
   return cudaGetLastError();

@@ -46,8 +46,8 @@ extern "C" {
 
 typedef enum {
   STARK_F64 = 0,            /* fp64 in/out; leaves of side >= 128 as fp16 digit        */
-                            /* products on the tensor cores with an accuracy proof per  */
-                            /* product, redone on the CUDA cores where it fails; other  */
+                            /* products on the tensor cores where they provably keep    */
+                            /* FP64's error bound, else redone on the CUDA cores; other */
                             /* leaves, depth-first and sharded plans on the CUDA cores  */
   STARK_F32_SPLIT_BF16 = 1, /* fp32 in/out; leaves as 3 bf16 products (hi*hi + hi*lo +  */
                             /* lo*hi, x = hi + lo) on tcgen05 tensor cores, fp32 accum. */
@@ -142,8 +142,11 @@ STARK_API stark_status stark_plan_get_info(stark_plan_t plan, stark_plan_info *i
  * combine (Alg. 5) adds each product into C with its signs.
  * A, B, C: device pointers to n x n matrices of the plan's
  * element type (double, float, float, int64_t).  C is overwritten; it may not
- * alias A or B.  Enqueues: zero C, divide A, divide B, one leaf-product launch
- * whose epilogue accumulates every leaf into C with the combine signs.
+ * alias A or B.  Enqueues the divide of A and B (which also clears C where
+ * leaves are added into it), one leaf-product launch, whose epilogue
+ * accumulates every leaf into C with the combine signs or stores its product,
+ * and for stored products the combine pass.  F64 products that digit products
+ * cannot prove accurate are redone by launches that otherwise do nothing.
  * Asynchronous on `stream`; capturable in a CUDA graph (no allocation, no
  * synchronisation).  n == 0 is a no-op. */
 STARK_API stark_status stark_mul(stark_plan_t plan, const void *A, const void *B, void *C, void *stream);
@@ -363,16 +366,18 @@ STARK_API stark_status stark_plan_check(stark_plan_t plan, void *stream);
  * stream.  stark_plan_set_timing(plan, k) pre-creates k event sets and
  * records the phases of the next k products (k = 0 switches timing off);
  * stark_plan_phase_ms waits for the last recorded product and returns the
- * mean over the recorded products of: [0] zeroing C, [1] divide A and B,
- * [2] leaf products with the fused combine.  Errors: EINVAL when nothing was
- * recorded. */
+ * mean over the recorded products of: [0] zeroing C by itself (near 0 where
+ * the divide clears C or nothing has to), [1] divide A and B, with the clearing
+ * of C for breadth-first products of the split dtypes, [2] leaf products with
+ * the fused combine.  Errors: EINVAL when nothing was recorded. */
 STARK_API stark_status stark_plan_set_timing(stark_plan_t plan, int records);
 STARK_API stark_status stark_plan_phase_ms(stark_plan_t plan, float out_ms[3]);
 
-/* The same means split one step further, `count` (1..4) of: [0] zeroing C,
- * [1] divide A and B, [2] the leaf-product kernel (with the fused combine,
- * when it is fused), [3] what follows it: the separate combine pass of
- * combine modes 2 and 3, the peeled edge and the staging copy into C (near 0
+/* The same means split one step further, `count` (1..4) of: [0] and [1] as
+ * above, [2] the leaf-product kernel (with the fused combine, when it is
+ * fused), [3] what follows it: the separate combine pass of combine modes 2
+ * and 3, of digit products and of bounded integers, the launches that redo an
+ * unproven F64 product, the peeled edge and the staging copy into C (near 0
  * when there is none).  Errors: EINVAL when nothing was recorded or count is
  * out of range. */
 STARK_API stark_status stark_plan_phases(stark_plan_t plan, float *out_ms, int count);
@@ -448,8 +453,10 @@ typedef struct stark_server_s *stark_server_t;
  * of the bytes; the fewest levels that fit; as stark_plan_set_traversal);
  * its requests run alone, subtree by subtree, not in the grouped launch.
  * When no traversal fits at the automatic depth, the fitting depth that the
- * cost model ranks fastest serves the request.  Thread-safe.  Errors: EINVAL (budget 0, slots outside 1..64),
- * EUNSUPPORTED, ENOMEM. */
+ * cost model ranks fastest serves the request.  F64 and I64 requests run alone,
+ * with their leaves on the CUDA cores at 8 bytes per operand element; their
+ * automatic depth is that path's, which may differ from a plan's.  Thread-safe.
+ * Errors: EINVAL (budget 0, slots outside 1..64), EUNSUPPORTED, ENOMEM. */
 STARK_API stark_status stark_server_create(size_t hbm_budget_bytes, int32_t slots, stark_server_t *out);
 
 /* How a server with `hbm_budget_bytes` would hold a request of side n, on

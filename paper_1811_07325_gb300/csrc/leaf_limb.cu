@@ -25,9 +25,9 @@
 //               keeps 88; 128 x 88 + 256 x 208 are the 384 x 168 of the launch).
 //               Each phase's diagonals are drained from TMEM, converted to
 //               int32 (exact) and added into a 64-bit running sum held in
-//               registers; after the last superchunk the sums
-//               (F64: rescaled and rounded once) are added into the leaf's C
-//               targets by bulk reductions.
+//               registers; after the last superchunk the sums (F64: rescaled
+//               and rounded once) are stored, for a whole product, or added into
+//               the leaf's C targets by atomics, for a range of its leaves.
 //
 // Order of the products.  TMEM holds four 128 x 128 accumulators, so K runs in
 // superchunks of 256 with three phases: twice, for each 128 of K, diagonals

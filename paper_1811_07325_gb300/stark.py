@@ -364,9 +364,9 @@ class Plan:
 
     def phase_ms(self):
         """Mean per-phase device time (ms) over the recorded products:
-        zeroing C, the divide, the leaf products with the combine, and that
-        last phase split into the leaf kernel and what follows it (the
-        separate combine pass of combine modes 2 and 3, peeled edge,
+        zeroing C by itself (near 0 where the divide clears it), the divide,
+        the leaf products with the combine, and that last phase split into the
+        leaf kernel and what follows it (a separate combine pass, peeled edge,
         staging copy)."""
         out = (ctypes.c_float * 4)()
         _check(_lib.stark_plan_phases(self._h, out, 4), "stark_plan_phases")

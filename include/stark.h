@@ -155,7 +155,9 @@ STARK_API stark_status stark_mul(stark_plan_t plan, const void *A, const void *B
  * into plan-owned buffers, runs stark_mul, copies C device->host and waits
  * for completion (then reports device-side errors like stark_plan_check).
  * A, B, C: host pointers (pinned memory gives full copy bandwidth).
- * Synchronous.  Allocates two staging sets (6 n^2 elements) on first use. */
+ * Synchronous.  Allocates two staging sets (6 n^2 elements) on first use; where
+ * they do not fit beside an F64 or I64 plan's digit planes, the plan gives those
+ * up and runs its leaves on the CUDA cores from then on. */
 STARK_API stark_status stark_mul_host(stark_plan_t plan, const void *A, const void *B, void *C, void *stream);
 
 /* Asynchronous form of stark_mul_host for streams of products: enqueues the

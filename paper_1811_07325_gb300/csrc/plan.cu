@@ -429,8 +429,7 @@ stark_status stark_mul_leaves(stark_plan_t p, const void* A, const void* B, void
 }
 
 // Staging buffers and pipeline streams for the host entry points.
-static stark_status ensure_host_pipeline(stark_plan_t p) {
-  if (p->ev_out[1]) return STARK_OK;  // created last: the whole pipeline exists
+static stark_status make_host_pipeline(stark_plan_t p) {
   // all or nothing: on any failure release what this call created
   const size_t bytes = (size_t)p->n * p->n * p->esz;
   void** bufs[6] = {&p->stage_A, &p->stage_B, &p->stage_C, &p->stage2[0], &p->stage2[1], &p->stage2[2]};
@@ -457,6 +456,19 @@ static stark_status ensure_host_pipeline(stark_plan_t p) {
       if (*e) cudaEventDestroy(*e);
       *e = nullptr;
     }
+  }
+  return st;
+}
+
+static stark_status plan_drop_limbs(stark_plan_s* p);
+
+static stark_status ensure_host_pipeline(stark_plan_t p) {
+  if (p->ev_out[1]) return STARK_OK;  // created last: the whole pipeline exists
+  stark_status st = make_host_pipeline(p);
+  if (st == STARK_ENOMEM && p->op_elem == 16) {
+    // the staging buffers come before the digit planes, which can do without
+    st = plan_drop_limbs(p);
+    if (st == STARK_OK) st = make_host_pipeline(p);
   }
   return st;
 }
@@ -853,6 +865,14 @@ static stark_status plan_alloc_operands(stark_plan_s* p, int64_t planes, bool wh
   if (st == STARK_ENOMEM) st = plan_alloc_operands_at(p, planes, half_split(p->dt) ? 4 : 8);
   if (st == STARK_OK && whole && p->int_tc) st = plan_int_products(p);
   return st;
+}
+
+// A plan with digit planes becomes one of 8 bytes per operand element for good.
+static stark_status plan_drop_limbs(stark_plan_s* p) {
+  if (cudaDeviceSynchronize() != cudaSuccess) return STARK_ECUDA;
+  p->limb_ok = false;
+  plan_free_products(p);
+  return plan_alloc_operands(p, p->P_ws, true);
 }
 
 stark_status stark_plan_set_traversal(stark_plan_t p, int levels) {
